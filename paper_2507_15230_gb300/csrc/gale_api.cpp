@@ -64,7 +64,6 @@ gale::Caps merge(const gale::Caps &a, const gale::Caps &b) {
     c.max_e = std::max(a.max_e, b.max_e);
     c.max_etv = std::max(a.max_etv, b.max_etv);
     c.max_tt = std::max(a.max_tt, b.max_tt);
-    c.max_up = std::max(a.max_up, b.max_up);
     c.hcap = std::max(a.hcap, b.hcap);
     c.n_tot = std::max(a.n_tot, b.n_tot);
     c.n_star = std::max(a.n_star, b.n_star);
@@ -110,7 +109,7 @@ gale_status plan_bins(gale_ctx *ctx, bool with_sizes) {
                                          " has a vertex with more than 255 upper neighbours (unsupported)");
         thr[k] = threads_for(ctx, ctx->hm.stats[k]);
         need[k] = gale::plan_smem(caps_k(k), thr[k]).total;
-        big[k] = need[k] > smem_cta;
+        big[k] = std::max<int64_t>(need[k], gale::class_bytes(caps_k(k), thr[k])) > smem_cta;
         if (k < K) cut[k] = ctx->hm.part_first[k + 1] > ctx->hm.part_first[k];
         if (with_sizes && k < K && size_t(k) < ctx->tt_general.size()) gen[k] = ctx->tt_general[k] != 0 && !big[k];
     }

@@ -149,39 +149,44 @@ struct Caps {
     int32_t max_e;      // largest owned edge count
     int32_t max_etv;    // largest sum of ET rows   (0 in counting plans)
     int32_t max_tt;     // largest sum of TT rows   (0 in counting plans)
-    int32_t max_up;     // most upper neighbours of an own vertex
     int32_t hcap;       // boundary-face hash capacity (power of two)
     int32_t n_tot;      // largest tet count of a block (external + internal + halo)
     int32_t n_star;     // largest external + internal tet count
 };
 
 // Byte offsets of the shared-memory regions of one CTA (all 16-aligned).
-// Two regions are reused from phase to phase:
-//   r2: VV and upper-endpoint staging, then the per-edge tet masks (which
-//       end up holding the ET row offsets);
-//   r1: VT per-warp counters and lane masks; then the neighbour bitmaps and
-//       their rank prefixes; then ET staging; then the boundary-face hash,
-//       the TT counts and the TT staging.
+// Some are reused from phase to phase:
+//   nbr: the stars in arrival order, each internal tet's edge ranks, then
+//       its TT links;
+//   jpos: positions in the VT rows, then every edge's first ET entry;
+//   r2: fill cursors, VV staging with the first ET entries and the list of long rows, then
+//       the per-edge tet masks;
+//   r1: the neighbour bitmaps and their rank prefixes; then ET staging; then
+//       the boundary-face hash, the TT counts and the TT staging.
+constexpr int32_t kKeyed = 1, kJpos16 = 2;
 struct SmemPlan {
     int32_t threads;
     int32_t W;          // row stride (words, odd) of the neighbour bitmaps
     int32_t nch;        // 32-tet chunks of the longest VT row
-    int32_t pad;        // per-warp counter row length (even)
-    int32_t scan;       // scan scratch (3 x 33 words)
+    int32_t stride;     // row stride of the padded rows (uint16s; 0: compact rows)
+    int32_t fill;       // the rows in arrival order (inside r2 and nbr)
+    int32_t mode;       // kKeyed: the rows' entries carry the vertex's slot in the tet;
+                        // kJpos16: VT rows may exceed 256 entries, positions are 16-bit
+    int32_t scan;       // scan scratch and flags
     int32_t blk;        // int32[blk_words] the cluster's block (bulk copy)
     int32_t vt_off;     // int32[nv_own+1]
     int32_t vt_list;    // uint16[n_vt]
-    int32_t c_vv;       // int32[nv_own+1] VV row offsets
+    int32_t c_vv;       // int32[nv_own+1] star counters, VV row offsets, edge bases
     int32_t c_e;        // int32[nv_own+1] first owned edge of each own vertex
     int32_t nbr;        // uint16[4*n_own] TT links
-    int32_t jpos;       // uint8 (or uint16 when jpos16)[4*n_star]: position of each
-                        // (tet, own slot) in that vertex's VT row
-    int32_t jpos16;     // 1: VT rows may exceed 256 entries, positions are 16-bit
+    int32_t jpos;       // uint8 (or uint16, kJpos16)[4*n_star]: position of each
+                        // (tet, own slot) in that vertex's VT row | int32[max_e]
     int32_t r2;         // uint16[max_vv] VV staging | uint32[max_e*nch] edge masks
-    int32_t st_w;       // uint16[max_e] upper-endpoint staging (inside r2)
+    int32_t et_b;       // int32[nv_own] first ET entries (inside r2)
+    int32_t long_rows;  // uint16[nv_own] vertices with more than 32 tets (inside r2)
     int32_t r1;         // see above
-    int32_t mk;         // phase B lane masks (inside r1)
     int32_t pre;        // uint8[nv_own*W] rank prefixes (inside r1)
+    int32_t ex;         // uint16[max_e] the edges' lower vertices (inside r1)
     int32_t tcnt;       // int32[n_own+1] TT counts (inside r1)
     int32_t st_tt;      // uint16[max_tt] TT staging (inside r1)
     int32_t total;      // bytes
@@ -202,10 +207,17 @@ SmemPlan plan_smem(const Caps &c, int threads);
 // Capacities of one cluster or part; staging capacities come from the exact
 // sizes of the counting pass (sizes == nullptr: a counting plan, no staging).
 Caps caps_of(const ClusterStat &s, const int64_t *sizes);
-// Shared memory a build plan of this working set would take at the given
-// block size, with its staging sized from estimates (the counting pass has
-// not run yet): used to decide which clusters to cut into parts.
-int64_t estimate_smem(const ClusterStat &s, int threads);
+// Size class of a working set, in bytes.  It draws the lines that callers
+// see: which clusters are cut into parts, and which run from global scratch
+// (and are refused by gale_build_clusters_noalloc).  It is the shared memory
+// of a build with counters and lane masks per warp in phase B; a build plan
+// near a CTA's limit (plan_smem) needs no more than that.
+int64_t class_bytes(const Caps &c, int threads);
+// ... with the staged rows' sizes from estimates (before the counting pass).
+int64_t estimate_class(const ClusterStat &s, int threads);
+
+// Padded rows are given up where the plan with them would pass this.
+constexpr int64_t kPaddedFit = 220 * 1024;
 
 // Size bins a context may have (one ticket counter each in the build and
 // serving paths).

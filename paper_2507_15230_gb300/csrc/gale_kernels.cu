@@ -12,24 +12,23 @@
 // except TT's rows of at most four entries, stored straight out.
 //
 //  B. VT (Section 4.6 / Algorithm 1: iterate the segment's tets and test
-//     each vertex against the segment interval).  Each warp takes a
-//     contiguous chunk of the tets (which are in canonical order) and counts
-//     its incidences per own vertex; a prefix across warps gives every
-//     (warp, vertex) its first slot, and within a warp the lanes holding the
-//     same vertex are ranked by a 32-bit lane mask.  Rows come out ascending
-//     with no sort.  (The paper's atomicPush, Algorithm 2, fills rows in
-//     arbitrary order.)
+//     each vertex against the segment interval): every incidence of an own
+//     vertex takes a slot of that vertex's row by one returning atomic (the
+//     paper's atomicPush, Algorithm 2), and the rows, in arrival order, are
+//     then sorted in registers: a thread sorts two rows of up to 32 tets at
+//     once, in the halves of 16-bit pairs, by a merge network.
 //  C. VV and the edges (x, w), x < w, that an own vertex x owns:
-//     - C1, per tet: the other vertices of every tet of VT(x) are ORed into
-//       a bitmap of x over the cluster's vertex universe; local order is
-//       canonical order, so the bitmap read in bit order is VV(x), sorted and
-//       deduplicated, and its bits above x are the upper endpoints w;
-//     - C2, per bitmap word: one block scan of the word popcounts places
-//       every VV row and every edge; each word keeps the rank of its first
-//       upper bit within its vertex, so an edge's index is one popcount away;
-//     - C3, per VT incidence (x, j-th tet of VT(x)): bit j is set in the tet
-//       mask of each edge (x, w) of that tet; a mask read in bit order is
-//       ET(x, w), ascending;
+//     - C1, in B's pass over the tets: the other vertices of every tet of
+//       VT(x) are ORed into a bitmap of x over the cluster's vertex universe;
+//       local order is canonical order, so the bitmap read in bit order is
+//       VV(x), sorted and deduplicated, and its bits above x are the upper
+//       endpoints w;
+//     - C2, per own vertex: the row lengths, four offsets by one block scan,
+//       and for each bitmap word the number of neighbours before it, so that
+//       an edge's index is one popcount away; then the VV rows, read out of
+//       the bitmaps while B's rows are sorted;
+//     - C3, per tet: bit j is set in the tet mask of each edge (x, w) of the
+//       tet, the j-th of VT(x); a mask read in bit order is ET(x, w);
 //     - C5, per internal tet (a, b, c, d): the AND of the masks of two edges
 //       (a, w1), (a, w2) holds the two tets of the face (a, w1, w2); the face
 //       (b, c, d) is matched the same way inside VT(b) when b is own;
@@ -47,6 +46,17 @@
 //
 // The counting mode runs the same passes without writes and returns the
 // exact sizes the host uses to place outputs and to admit cache entries.
+//
+// What bounds it: nothing here is a contraction, and DRAM is busy for a
+// fifth of the time.  The time follows the warp instructions of a cluster
+// (about 0.011 ms per thousand at 128^3, over every phase), with the shared-
+// memory pipe close behind, so the passes above are chosen for few
+// instructions per incidence.  Measured at 268 vertices / 1,536 tets a
+// cluster (2 CTAs of 512 threads an SM): 70.7k warp instructions and 24.4k
+// wavefronts, 7.06 ms per 256^3 build; with a stable fill from per-warp
+// counters and lane masks in B, C1 as a pass of its own, edge ranks
+// recomputed in C5 and a scan over the edges in C4 it was 107.6k, 29.8k and
+// 9.07 ms.
 #include <cuda_runtime.h>
 #include <stdint.h>
 
@@ -60,6 +70,10 @@ namespace gale {
 
 namespace {
 
+// scan scratch: block_scan4's words, and four flags in those that blocks of
+// up to 27 warps leave free
+constexpr int scan_words(int threads) { return threads <= 864 ? 128 : 140; }
+GALE_HD constexpr int flag_word(int warps) { return warps <= 27 ? 28 : 136; }
 constexpr unsigned FULL = 0xffffffffu;
 constexpr int kWaitLimit = 1 << 22;  // polls of the block copy's barrier before giving up
 
@@ -69,19 +83,21 @@ struct Smem {
     int32_t *vt_off;
     uint16_t *vt_list;
     int32_t *c_vv, *c_e;
+    uint16_t *fill;       // r2 and nbr
     uint16_t *nbr;
-    uint8_t *jpos;
-    uint32_t *emask;  // r2
-    uint16_t *st_v;   // r2
-    uint16_t *st_w;   // r2
-    uint16_t *cw;     // r1 (phase B)
-    uint32_t *mk;     // r1 (phase B)
-    uint32_t *bm;     // r1 (phase C)
-    uint8_t *pre;     // r1 (phase C)
-    uint16_t *st_et;  // r1 (phase C4)
-    uint32_t *hash;   // r1 (phase D)
-    int32_t *tcnt;    // r1 (phases D, E)
-    uint16_t *st_tt;  // r1 (phase E)
+    uint8_t *jpos;        // until C5
+    int32_t *eo;          // jpos (phase C4)
+    uint32_t *emask;      // r2
+    uint16_t *st_v;       // r2
+    int32_t *et_b;        // r2
+    uint16_t *long_rows;  // r2
+    uint32_t *bm;         // r1 (until C3)
+    uint8_t *pre;         // r1 (until C3)
+    uint16_t *st_et;      // r1 (phase C4)
+    uint16_t *ex;         // r1 (phase C4)
+    uint32_t *hash;       // r1 (phase D)
+    int32_t *tcnt;        // r1 (phases D, E)
+    uint16_t *st_tt;      // r1 (phase E')
 };
 
 __device__ __forceinline__ Smem carve(char *base, const SmemPlan &p) {
@@ -92,16 +108,18 @@ __device__ __forceinline__ Smem carve(char *base, const SmemPlan &p) {
     s.vt_list = reinterpret_cast<uint16_t *>(base + p.vt_list);
     s.c_vv = reinterpret_cast<int32_t *>(base + p.c_vv);
     s.c_e = reinterpret_cast<int32_t *>(base + p.c_e);
+    s.fill = reinterpret_cast<uint16_t *>(base + p.fill);
     s.nbr = reinterpret_cast<uint16_t *>(base + p.nbr);
     s.jpos = reinterpret_cast<uint8_t *>(base + p.jpos);
+    s.eo = reinterpret_cast<int32_t *>(base + p.jpos);
     s.emask = reinterpret_cast<uint32_t *>(base + p.r2);
     s.st_v = reinterpret_cast<uint16_t *>(base + p.r2);
-    s.st_w = reinterpret_cast<uint16_t *>(base + p.st_w);
-    s.cw = reinterpret_cast<uint16_t *>(base + p.r1);
-    s.mk = reinterpret_cast<uint32_t *>(base + p.mk);
+    s.et_b = reinterpret_cast<int32_t *>(base + p.et_b);
+    s.long_rows = reinterpret_cast<uint16_t *>(base + p.long_rows);
     s.bm = reinterpret_cast<uint32_t *>(base + p.r1);
     s.pre = reinterpret_cast<uint8_t *>(base + p.pre);
     s.st_et = reinterpret_cast<uint16_t *>(base + p.r1);
+    s.ex = reinterpret_cast<uint16_t *>(base + p.ex);
     s.hash = reinterpret_cast<uint32_t *>(base + p.r1);
     s.tcnt = reinterpret_cast<int32_t *>(base + p.tcnt);
     s.st_tt = reinterpret_cast<uint16_t *>(base + p.st_tt);
@@ -211,36 +229,36 @@ __device__ __forceinline__ int block_scan_thread(const Team &tm, int v, int32_t 
     return scr[warp] + incl - v;
 }
 
-// Exclusive scans of three values per thread over the team, in place;
-// totals to t[0..2].  scr needs 99 words.  Ends synced.
+// Exclusive scans of four values per thread over the team, in place; totals
+// to t[0..3].  scr needs 128 words (136 with 32 warps).
 template <class Team>
-__device__ __forceinline__ void block_scan3(const Team &tm, int &a, int &b, int &c, int32_t *scr, int *t) {
+__device__ __forceinline__ void block_scan4(const Team &tm, int &a, int &b, int &c, int &d, int32_t *scr, int *t) {
     const int nw = tm.nt() >> 5;
     const int lane = tm.tid() & 31, warp = tm.tid() >> 5;
-    const int ia = warp_incl_scan(a, lane), ib = warp_incl_scan(b, lane), ic = warp_incl_scan(c, lane);
+    int32_t *const tot = nw < 32 ? scr + nw : scr + 128;
+    const int ts = nw < 32 ? 32 : 1;
+    const int ia = warp_incl_scan(a, lane), ib = warp_incl_scan(b, lane);
+    const int ic = warp_incl_scan(c, lane), id = warp_incl_scan(d, lane);
     if (lane == 31) {
         scr[warp] = ia;
-        scr[33 + warp] = ib;
-        scr[66 + warp] = ic;
+        scr[32 + warp] = ib;
+        scr[64 + warp] = ic;
+        scr[96 + warp] = id;
     }
     tm.sync();
-    if (warp == 0) {
+    for (int s = warp; s < 4; s += nw) {  // a warp per value
+        const int w = lane < nw ? scr[32 * s + lane] : 0;
+        const int wi = warp_incl_scan(w, lane);
+        if (lane < nw) scr[32 * s + lane] = wi - w;
+        if (lane == 31) tot[ts * s] = wi;
+    }
+    tm.sync();
 #pragma unroll
-        for (int s = 0; s < 3; ++s) {
-            const int w = lane < nw ? scr[33 * s + lane] : 0;
-            const int wi = warp_incl_scan(w, lane);
-            if (lane < nw) scr[33 * s + lane] = wi - w;
-            if (lane == 31) scr[33 * s + 32] = wi;
-        }
-    }
-    tm.sync();
-    t[0] = scr[32];
-    t[1] = scr[65];
-    t[2] = scr[98];
+    for (int s = 0; s < 4; ++s) t[s] = tot[ts * s];
     a = scr[warp] + ia - a;
-    b = scr[33 + warp] + ib - b;
-    c = scr[66 + warp] + ic - c;
-    tm.sync();
+    b = scr[32 + warp] + ib - b;
+    c = scr[64 + warp] + ic - c;
+    d = scr[96 + warp] + id - d;
 }
 
 // p[0 .. n) = v over the team, 16 bytes a store (p is 16-byte aligned: every
@@ -297,18 +315,10 @@ __device__ int block_scan_array(const Team &tm, int32_t *a, int n, int32_t *scr)
     return total;
 }
 
-// The face of a packed row opposite slot s: the other three 16-bit ids,
-// ascending, packed into 48 bits.
-__device__ __forceinline__ uint64_t face_key(uint2 r, int s) {
-    const uint64_t row = uint64_t(r.x) | (uint64_t(r.y) << 32);
-    const int sh = 16 * s;
-    const uint64_t low = sh ? (row & ((uint64_t(1) << sh) - 1)) : 0ull;
-    const uint64_t high = s == 3 ? 0ull : ((row >> (sh + 16)) << sh);
-    return low | high;
-}
-
-__device__ __forceinline__ uint32_t face_hash(uint64_t key, uint32_t mask) {
-    return uint32_t((key * 0x9E3779B97F4A7C15ull) >> 40) & mask;
+// Hash of a face, its three 16-bit ids as (first, second | third << 16).
+__device__ __forceinline__ uint32_t face_hash(uint2 key) {
+    const uint32_t h = key.y * 0x9E3779B1u + key.x * 0x85EBCA77u;
+    return h ^ (h >> 15);
 }
 
 // number of local vertex ids two packed rows have in common
@@ -334,10 +344,132 @@ __device__ __forceinline__ void cswap2(int32_t &a, int32_t &b, uint32_t &pa, uin
     pb = qb;
 }
 
-// hash entries: bits [0, 20) = 4 * internal-tet index + slot + 1, bits
-// [20, 32) = number of other tets matched to the face
-constexpr uint32_t kRefMask = (1u << 20) - 1u;
-constexpr uint32_t kMatch = 1u << 20;
+// hash entries: bits [0, 17) = internal-tet index + 1, bits [17, 32) =
+// number of other tets matched to the face
+constexpr uint32_t kRefMask = (1u << 17) - 1u;
+constexpr uint32_t kMatch = 1u << 17;
+
+template <int N>
+struct IntC {
+    static constexpr int value = N;
+};
+
+// stars larger than this count their tets and ET entries in two words
+constexpr int32_t kMaxPacked = 21845;
+constexpr int kOffMask = 0xffffff;  // VV offsets (at most 6 x 65534) under the 8-bit bias
+
+__device__ __forceinline__ void cmpx_u16x2(uint32_t &a, uint32_t &b) {
+    uint32_t lo, hi;
+    asm("min.u16x2 %0, %1, %2;" : "=r"(lo) : "r"(a), "r"(b));
+    asm("max.u16x2 %0, %1, %2;" : "=r"(hi) : "r"(a), "r"(b));
+    a = lo;
+    b = hi;
+}
+
+// one row of a star: n entries from `in`, written in order from `out`
+struct SortRow {
+    int n, in, out;
+};
+
+// Two rows of up to N distinct 16-bit entries each, sorted by one thread in
+// registers: row a in the low halves, row b in the high ones (Batcher's
+// odd-even merge network, pruned to N).  N = 64: one row of 33 to 64 entries
+// (b is its tail from the 33rd), whose sorted halves a bitonic merge then
+// joins.  Input rows start on a word and are padded with 0xffff to one.
+// keyed: entries are 4 * tet + slot; the tets go out, and every entry's
+// position goes to jpos (16-bit with jp16).
+template <int N>
+__device__ __forceinline__ void sort_rows(const uint16_t *in, uint16_t *out, uint8_t *jpos, bool keyed, bool jp16,
+                                          const SortRow &a, const SortRow &b) {
+    constexpr int R = N < 32 ? N : 32;
+    uint32_t v[R];
+    const uint32_t *wa = reinterpret_cast<const uint32_t *>(in + a.in);
+    const uint32_t *wb = reinterpret_cast<const uint32_t *>(in + b.in);
+#pragma unroll
+    for (int i = 0; i < R; i += 2) {
+        const uint32_t x = i < a.n ? wa[i >> 1] : 0xffffffffu, y = i < b.n ? wb[i >> 1] : 0xffffffffu;
+        v[i] = __byte_perm(x, y, 0x5410);
+        v[i + 1] = __byte_perm(x, y, 0x7632);
+    }
+#pragma unroll
+    for (int p = 1; p < R; p <<= 1)
+#pragma unroll
+        for (int k = p; k >= 1; k >>= 1)
+#pragma unroll
+            for (int i = 0; i + k < R; ++i)
+                if (i >= k % p && ((i - k % p) / k) % 2 == 0 && i / (2 * p) == (i + k) / (2 * p))
+                    cmpx_u16x2(v[i], v[i + k]);
+    if (N == 64) {
+#pragma unroll
+        for (int i = 0; i < R / 2; ++i) {  // low[i] against high[31 - i], and high[i] against low[31 - i]
+            uint32_t lo = v[i], hi = (v[R - 1 - i] >> 16) | (v[R - 1 - i] << 16);
+            cmpx_u16x2(lo, hi);
+            v[i] = (lo & 0xffffu) | (hi << 16);
+            v[R - 1 - i] = (lo >> 16) | (hi & 0xffff0000u);
+        }
+#pragma unroll
+        for (int k = R / 2; k >= 1; k >>= 1)
+#pragma unroll
+            for (int i = 0; i < R; ++i)
+                if ((i & k) == 0) cmpx_u16x2(v[i], v[i + k]);
+    }
+    uint16_t *const oa = out + a.out, *const ob = out + b.out;
+    if (keyed && !jp16) {
+#pragma unroll
+        for (int i = 0; i < R; ++i) {
+            const uint32_t x = v[i] & 0xffffu, y = v[i] >> 16;
+            if (i < a.n) {
+                oa[i] = uint16_t(x >> 2);
+                jpos[x] = uint8_t(i);
+            }
+            if (i < b.n) {
+                ob[i] = uint16_t(y >> 2);
+                jpos[y] = uint8_t(N == 64 ? i + 32 : i);
+            }
+        }
+        return;
+    }
+    auto put = [&](uint16_t *o, int i, int pos, uint32_t e) {
+        o[i] = uint16_t(keyed ? e >> 2 : e);
+        if (keyed) reinterpret_cast<uint16_t *>(jpos)[e] = uint16_t(pos);
+    };
+#pragma unroll
+    for (int i = 0; i < R; ++i) {
+        if (i < a.n) put(oa, i, i, v[i] & 0xffffu);
+        if (i < b.n) put(ob, i, N == 64 ? i + 32 : i, v[i] >> 16);
+    }
+}
+
+// One row of any length sorted in place by a warp: a bitonic network whose
+// comparisons all point the same way, so that the pairs past the end drop out.
+__device__ __forceinline__ void sort_row_warp(uint16_t *v, int n, int lane) {
+    int half = 32;
+    while (2 * half < n) half <<= 1;
+    auto cx = [&](int a, int b) {
+        if (b < n) {
+            const uint16_t x = v[a], y = v[b];
+            if (y < x) {
+                v[a] = y;
+                v[b] = x;
+            }
+        }
+    };
+    for (int k = 2; (k >> 1) < n; k <<= 1) {
+        const int kh = k >> 1;
+        for (int i = lane; i < half; i += 32) {
+            const int a = (i & ~(kh - 1)) * 2, f = i & (kh - 1);
+            cx(a + f, a + k - 1 - f);
+        }
+        __syncwarp();
+        for (int j = kh >> 1; j > 0; j >>= 1) {
+            for (int i = lane; i < half; i += 32) {
+                const int a = (i & ~(j - 1)) * 2 + (i & (j - 1));
+                cx(a, a + j);
+            }
+            __syncwarp();
+        }
+    }
+}
 
 // ---------------- E'. TT of a non-manifold cluster ----------------
 // A triangle of the block lies in three or more tets, so a face may have
@@ -422,8 +554,8 @@ __device__ bool run_cluster(const Team &tm, const DevMesh &m, const SmemPlan &pl
     const uint32_t lt = (1u << lane) - 1u;
     const Caps &caps = plan.caps;
     const int32_t *__restrict__ g = m.blocks + blk_word;
-    int32_t *flag = S.scan + 120;  // [0] block fits, [1] bulk copy issued, [2] non-manifold
-    const bool jp16 = plan.jpos16 != 0;
+    int32_t *flag = S.scan + flag_word(NWARP);  // [0] block fits, [1] bulk copy issued, [2] non-manifold, [3] long rows
+    const bool jp16 = (plan.mode & kJpos16) != 0;
 
     // ---------------- A. the block, by one bulk copy ----------------
     if (tid == 0) {
@@ -436,6 +568,7 @@ __device__ bool run_cluster(const Team &tm, const DevMesh &m, const SmemPlan &pl
         flag[0] = fits;
         flag[1] = issued;
         flag[2] = 0;
+        flag[3] = 0;
     }
     tm.sync();
     const bool fits = flag[0] != 0, issued = flag[1] != 0;
@@ -490,11 +623,20 @@ __device__ bool run_cluster(const Team &tm, const DevMesh &m, const SmemPlan &pl
     const bool do_et = !COUNT && (mask & R_ET);
     const int32_t t_base = h.t_base;
     const int n_halo_b = h.n_halo;
-    // canonical id of a local tet
+    // canonical id of a local tet: of the star tets (external and internal)
+    // by one predicated load, of any tet by two
+    const int32_t t_own = t_base - n_ext;
+    auto gstar = [&](int loc) -> int32_t {
+        if (PART) return tmap[loc < n_ext ? loc : n_halo_b + loc];
+        int32_t g1 = loc + t_own;
+        if (loc < n_ext) g1 = tmap[loc];
+        return g1;
+    };
     auto gtet = [&](int loc) -> int32_t {
-        if (loc < n_ext) return tmap[loc];
-        if (loc < n_vtets) return part ? tmap[n_halo_b + loc] : t_base + (loc - n_ext);
-        return tmap[loc - n_own];
+        if (PART) return loc >= n_vtets ? tmap[loc - n_own] : gstar(loc);
+        int32_t g1 = loc + t_own;
+        if (uint32_t(loc - n_ext) >= uint32_t(n_own)) g1 = tmap[loc < n_ext ? loc : loc - n_own];
+        return g1;
     };
     // a part writes cluster-level offset values: its entries are shifted by
     // those of the cluster's earlier parts
@@ -506,408 +648,486 @@ __device__ bool run_cluster(const Team &tm, const DevMesh &m, const SmemPlan &pl
         b_et = __ldg(&part->b_et);
     }
 
-    // The per-own-vertex passes of C2 leave whole warps idle when the cluster
-    // has fewer own vertices than the block has threads less a warp: those
-    // warps copy VT out meanwhile (vt_off and vt_list do not change after B).
-    const int copy_warp0 = (nvo + 31) >> 5;
-    const bool vt_copy_later = !COUNT && (mask & R_VT) && copy_warp0 < NWARP &&
-                               (COUNT || (mask & (R_VV | R_ET | R_TT)));
-
-    // ---------------- B. VT ----------------
-    int vt_total;
-    {
-        const int pad = plan.pad;
-        uint16_t *cw = S.cw;  // [warp][v]: counts, then next position within the row
-        uint32_t *cw32 = reinterpret_cast<uint32_t *>(S.cw);
-        uint32_t *mk = S.mk;  // [warp][v]: lanes holding v
-        const int chunk = ((n_vtets + NWARP - 1) / NWARP + 31) & ~31;
-        const int c0 = min(n_vtets, warp * chunk), c1 = min(n_vtets, c0 + chunk);
-        fill_words(tm, cw32, (NWARP * pad) >> 1, 0u);  // pad is even
-        fill_words(tm, mk, NWARP * pad, 0u);
-        tm.sync();
-        for (int i = c0 + lane; i < c1; i += 32) {
-            const uint2 r = rows[i];
-#pragma unroll
-            for (int s = 0; s < 4; ++s) {
-                const uint32_t d = vtx(r, s) - uint32_t(lo);
-                if (d < nvo_u) atomicAdd(&cw32[(warp * pad + int(d)) >> 1], 1u << (16 * (d & 1u)));
-            }
-        }
-        tm.sync();
-        // row lengths -> offsets; every (warp, vertex) gets its first position
-        for (int v = tid; v < nvo; v += NT) {
-            int tot = 0;
-            for (int w = 0; w < NWARP; ++w) tot += int(cw[w * pad + v]);
-            S.vt_off[v] = tot;
-        }
-        tm.sync();
-        vt_total = block_scan_array(tm, S.vt_off, nvo, S.scan);
-        bool bad = vt_total > caps.n_vt;
-        for (int v = tid; v < nvo; v += NT) {
-            const int d = (v + 1 < nvo ? S.vt_off[v + 1] : vt_total) - S.vt_off[v];
-            bad |= d > caps.max_deg;
-            int run = 0;
-            for (int w = 0; w < NWARP; ++w) {
-                const int c = int(cw[w * pad + v]);
-                cw[w * pad + v] = uint16_t(run);
-                run += c;
-            }
-        }
-        if (tid == 0) S.vt_off[nvo] = vt_total;
-        if (tm.sync_or(bad)) {
-            if (tid == 0) atomicOr(err, ERR_CAPACITY);
-            return true;
-        }
-        // fill in tet order, 32 tets per step of each warp; the position
-        // of every (tet, own vertex) in that vertex's row is kept for C3/C5
-        for (int i0 = c0; i0 < c1; i0 += 32) {
-            const int i = i0 + lane;
-            const uint2 r = i < c1 ? rows[i] : make_uint2(0xffffffffu, 0xffffffffu);
-            uint32_t d[4];
-#pragma unroll
-            for (int s = 0; s < 4; ++s) {
-                d[s] = vtx(r, s) - uint32_t(lo);
-                if (d[s] < nvo_u) atomicOr(&mk[warp * pad + d[s]], 1u << lane);
-            }
-            __syncwarp();
-            uint32_t mm[4];
-#pragma unroll
-            for (int s = 0; s < 4; ++s) {
-                mm[s] = 0u;
-                if (d[s] < nvo_u) {
-                    mm[s] = mk[warp * pad + d[s]];
-                    const int pos = int(cw[warp * pad + d[s]]) + __popc(mm[s] & lt);
-                    S.vt_list[S.vt_off[d[s]] + pos] = uint16_t(i);
-                    if (jp16) reinterpret_cast<uint16_t *>(S.jpos)[4 * i + s] = uint16_t(pos);
-                    else S.jpos[4 * i + s] = uint8_t(pos);
-                }
-            }
-            __syncwarp();
-#pragma unroll
-            for (int s = 0; s < 4; ++s)
-                if (d[s] < nvo_u && (mm[s] & lt) == 0u) {
-                    cw[warp * pad + d[s]] += uint16_t(__popc(mm[s]));
-                    mk[warp * pad + d[s]] = 0u;
-                }
-            __syncwarp();
-        }
-        tm.sync();
-        if (COUNT) {
-            if (tid == 0) sizes_out[SZ_VT] = vt_total;
-        } else if ((mask & R_VT) && !vt_copy_later) {
-            for (int i = tid; i <= nvo; i += NT) it->vt_off[i] = S.vt_off[i] + b_vt;
-            copy_out(tm, it->vt_val, vt_total, [&](int j) { return gtet(S.vt_list[j]); });
-        }
-    }
-    if (!(COUNT || do_vv || do_et || want_tt)) return true;
-
-    // ---------------- C1. neighbour bitmaps, per tet ----------------
+    const bool need_nb = COUNT || do_vv || do_et || want_tt;
     const int W = (h.nv_nb + 31) >> 5;  // bitmap words per vertex
     const int WP = W | 1;                // row stride (odd: rows start in different banks)
     uint32_t *bm = S.bm;
     uint8_t *pre = S.pre;
-    fill_words(tm, bm, nvo * WP, 0u);
-    if (want_tt) {
-        uint32_t *nb32 = reinterpret_cast<uint32_t *>(S.nbr);
-        fill_words(tm, nb32, 2 * n_own, FULL);
+
+    // ---------------- B/C1. stars and neighbour bitmaps, per tet ----------
+    // For every own vertex x of a tet: one atomic counts x's star (low half
+    // of the counter) and the ET entries x owns (high half: a tet gives x
+    // one for each of its vertices above x), and the other three vertices
+    // are ORed into x's bitmap.  With padded rows (plan.stride) the value the
+    // count returns is also the tet's slot; otherwise a second pass fills
+    // compact rows by cursors.  An entry is 4 * tet + x's slot in the tet
+    // (kKeyed).
+    int32_t *const cnt = S.c_vv;  // the counters, then VV offsets, then the biased edge bases
+    int32_t *const et_b = S.et_b;  // first ET entry of each own vertex
+    const int stride = plan.stride;
+    const bool keyed = (plan.mode & kKeyed) != 0, wide = caps.max_deg > kMaxPacked;
+    uint16_t *const fill = S.fill;  // rows in arrival order, each from a word boundary
+    int32_t *const cur = reinterpret_cast<int32_t *>(S.st_v);  // fill cursors of compact rows
+    auto row_at = [&](int x) -> int { return stride ? x * stride : (S.vt_off[x] + x + 1) & ~1; };
+    int32_t flags = 0;
+    for (int i = tid; i <= nvo; i += NT) {
+        cnt[i] = 0;
+        S.vt_off[i] = 0;
     }
+    if (need_nb) fill_words(tm, bm, nvo * WP, 0u);
+    fill_words(tm, reinterpret_cast<uint32_t *>(fill), stride ? (nvo * stride) >> 1 : (caps.n_vt + nvo + 3) >> 1, FULL);
     tm.sync();
-    int etv = 0;  // ET entries: each own vertex of a tet, once per vertex above it
     for (int i = tid; i < n_vtets; i += NT) {
         const uint2 r = rows[i];
-        const uint32_t v0 = r.x & 0xffffu, v1 = r.x >> 16, v2 = r.y & 0xffffu, v3 = r.y >> 16;
-        uint32_t d = v0 - uint32_t(lo);
-        if (d < nvo_u) {
-            uint32_t *row = bm + d * WP;
-            atomicOr(row + (v1 >> 5), 1u << (v1 & 31));
-            atomicOr(row + (v2 >> 5), 1u << (v2 & 31));
-            atomicOr(row + (v3 >> 5), 1u << (v3 & 31));
-            etv += 3;
+        const uint32_t v[4] = {r.x & 0xffffu, r.x >> 16, r.y & 0xffffu, r.y >> 16};
+        uint32_t bit[4], q[4];
+#pragma unroll
+        for (int s = 0; s < 4; ++s) {
+            q[s] = v[s] >> 5;
+            bit[s] = 1u << (v[s] & 31u);
         }
-        d = v1 - uint32_t(lo);
-        if (d < nvo_u) {
-            uint32_t *row = bm + d * WP;
-            atomicOr(row + (v0 >> 5), 1u << (v0 & 31));
-            atomicOr(row + (v2 >> 5), 1u << (v2 & 31));
-            atomicOr(row + (v3 >> 5), 1u << (v3 & 31));
-            etv += 2;
-        }
-        d = v2 - uint32_t(lo);
-        if (d < nvo_u) {
-            uint32_t *row = bm + d * WP;
-            atomicOr(row + (v0 >> 5), 1u << (v0 & 31));
-            atomicOr(row + (v1 >> 5), 1u << (v1 & 31));
-            atomicOr(row + (v3 >> 5), 1u << (v3 & 31));
-            etv += 1;
-        }
-        d = v3 - uint32_t(lo);
-        if (d < nvo_u) {
-            uint32_t *row = bm + d * WP;
-            atomicOr(row + (v0 >> 5), 1u << (v0 & 31));
-            atomicOr(row + (v1 >> 5), 1u << (v1 & 31));
-            atomicOr(row + (v2 >> 5), 1u << (v2 & 31));
+#pragma unroll
+        for (int s = 0; s < 4; ++s) {
+            const uint32_t d = v[s] - uint32_t(lo);
+            if (d < nvo_u) {
+                if (wide) {  // the halves could overflow: two counters
+                    atomicAdd(&cnt[d], 3 - s);
+                    atomicAdd(&S.vt_off[d + 1], 1);
+                } else {
+                    const int slot = atomicAdd(&cnt[d], 1 | ((3 - s) << 16)) & 0xffff;
+                    if (stride && slot < stride) fill[d * stride + slot] = uint16_t(keyed ? 4 * i + s : i);
+                }
+                if (need_nb) {
+                    uint32_t *row = bm + d * WP;
+#pragma unroll
+                    for (int u = 1; u < 4; ++u) atomicOr(row + q[(s + u) & 3], bit[(s + u) & 3]);
+                }
+            }
         }
     }
     tm.sync();
 
-    // ---------------- C2. VV rows and owned edges, per own vertex ----------
-    int tot[3];  // VV entries, owned edges, ET entries
+    // ---------------- C2. row lengths and offsets, per own vertex ----------
+    // Every bitmap word gets the number of neighbours before it (8 bits); the
+    // edge to y, one of x's upper neighbours, is then
+    //   base[x] + ((pre + popc(bits of y's word below y)) & 255),
+    // base being x's first edge less its lower neighbours (with more than 255
+    // neighbours the prefixes start from minus the lower ones instead).
+    int vt_total, et_total, vv_total = 0, tot_e = 0;
     {
-        // counts per vertex
-        for (int x = tid; x < nvo; x += NT) {
-            const uint32_t *row = bm + x * WP;
-            const int X = lo + x, qx = X >> 5;
-            const uint32_t hb = (X & 31) == 31 ? 0u : (FULL << ((X & 31) + 1));
-            int cv = 0, ce = 0;
-            for (int q = 0; q < W; ++q) {
-                const uint32_t w = row[q];
-                cv += __popc(w);
-                ce += __popc(w & (q < qx ? 0u : (q > qx ? FULL : hb)));
+        const int per = range_len(tm, nvo);
+        const int x0 = min(nvo, tid * per), x1 = min(nvo, x0 + per);
+        int sv = 0, se = 0, sn = 0, su = 0;
+        for (int x = x0; x < x1; ++x) {
+            const uint32_t c = uint32_t(cnt[x]);
+            const int d = wide ? S.vt_off[x + 1] : int(c & 0xffffu);
+            const int et = wide ? int(c) : int(c >> 16);
+            S.vt_off[x + 1] = d;
+            et_b[x] = et;
+            sv += d;
+            se += et;
+            if (d > caps.max_deg) flags |= ERR_CAPACITY;
+            if (need_nb) {
+                const uint32_t *row = bm + x * WP;
+                uint8_t *prx = pre + x * WP;
+                int n = 0;
+#pragma unroll 4
+                for (int q = 0; q < W; ++q) {
+                    prx[q] = uint8_t(n);
+                    n += __popc(row[q]);
+                }
+                const int X = lo + x, qx = X >> 5;
+                const uint32_t below = (1u << (X & 31)) - 1u;
+                int k0 = prx[qx] + __popc(row[qx] & below);  // neighbours below x
+                int bias = k0;
+                if (n > 255) {
+                    k0 = 0;
+                    for (int q = 0; q < qx; ++q) k0 += __popc(row[q]);
+                    k0 += __popc(row[qx] & below);
+                    int run = -k0;
+                    for (int q = 0; q < W; ++q) {
+                        prx[q] = uint8_t(run);
+                        run += __popc(row[q]);
+                    }
+                    bias = 0;
+                }
+                if (n - k0 > 255) flags |= ERR_CAPACITY;
+                S.c_vv[x] = n | int(uint32_t(bias) << 24);
+                S.c_e[x] = n - k0;
+                sn += n;
+                su += n - k0;
             }
-            S.c_vv[x] = cv;
-            S.c_e[x] = ce;
         }
-        tm.sync();
-        // exclusive scans of both count arrays, and the ET total
-        {
-            const int per = range_len(tm, nvo);
-            const int x0 = min(nvo, tid * per), x1 = min(nvo, x0 + per);
-            int sv = 0, se = 0;
-            for (int x = x0; x < x1; ++x) {
-                sv += S.c_vv[x];
-                se += S.c_e[x];
-            }
-            int et0 = etv;
-            block_scan3(tm, sv, se, et0, S.scan, tot);
-            for (int x = x0; x < x1; ++x) {
-                const int a = S.c_vv[x], b = S.c_e[x];
-                S.c_vv[x] = sv;
-                S.c_e[x] = se;
-                sv += a;
-                se += b;
-            }
-            if (tid == 0) {
-                S.c_vv[nvo] = tot[0];
-                S.c_e[nvo] = tot[1];
+        int tot[4];
+        block_scan4(tm, sv, se, sn, su, S.scan, tot);
+        vt_total = tot[0];
+        et_total = tot[1];
+        vv_total = tot[2];
+        tot_e = tot[3];
+        if (vt_total > caps.n_vt || tot_e > caps.max_e || ((do_vv || do_et) && vv_total > caps.max_vv) ||
+            (do_et && et_total > caps.max_etv))
+            flags |= ERR_CAPACITY;
+        for (int x = x0; x < x1; ++x) {
+            const int d = S.vt_off[x + 1], et = et_b[x];
+            if (d > 32) S.long_rows[atomicAdd(&flag[3], 1)] = uint16_t(x);
+            S.vt_off[x + 1] = sv + d;
+            if (!stride) cur[x] = (sv + x + 1) & ~1;
+            et_b[x] = se;
+            sv += d;
+            se += et;
+            if (need_nb) {
+                const int n = S.c_vv[x], u = S.c_e[x];
+                S.c_vv[x] = sn | (n & int(0xff000000u));  // the bias stays on top
+                S.c_e[x] = su;
+                sn += n & kOffMask;
+                su += u;
             }
         }
-        if (tot[1] > caps.max_e || (do_vv && tot[0] > caps.max_vv) || (do_et && tot[2] > caps.max_etv)) {
+        if (tid == 0) {
+            S.c_vv[nvo] = vv_total;
+            S.c_e[nvo] = tot_e;
+        }
+        if (tm.sync_or(flags)) {
             if (tid == 0) atomicOr(err, ERR_CAPACITY);
             return true;
         }
-        tm.sync();
-        if (vt_copy_later && warp >= copy_warp0) {
-            // VT out, on the warps the per-vertex loop below leaves idle
-            const int t0 = tid - copy_warp0 * 32, nt = NT - copy_warp0 * 32;
-            for (int i = t0; i <= nvo; i += nt) it->vt_off[i] = S.vt_off[i] + b_vt;
-            int j = t0;
-            for (; j + 3 * nt < vt_total; j += 4 * nt) {
-                const int32_t a = gtet(S.vt_list[j]), b = gtet(S.vt_list[j + nt]);
-                const int32_t c = gtet(S.vt_list[j + 2 * nt]), d = gtet(S.vt_list[j + 3 * nt]);
-                it->vt_val[j] = a;
-                it->vt_val[j + nt] = b;
-                it->vt_val[j + 2 * nt] = c;
-                it->vt_val[j + 3 * nt] = d;
+    }
+    if (!stride) {
+        for (int i = tid; i < n_vtets; i += NT) {
+            const uint2 r = rows[i];
+#pragma unroll
+            for (int s = 0; s < 4; ++s) {
+                const uint32_t d = vtx(r, s) - uint32_t(lo);
+                if (d < nvo_u) fill[atomicAdd(&cur[d], 1)] = uint16_t(keyed ? 4 * i + s : i);
             }
-            for (; j < vt_total; j += nt) it->vt_val[j] = gtet(S.vt_list[j]);
         }
-        // rows: one loop step per set bit, words visited through an
-        // occupancy mask; the word holding x keeps its upper bits only and
-        // every word with upper bits records the rank of its first one
-        bool bad = false;
-        for (int x = tid; x < nvo; x += NT) {
-            uint32_t *row = bm + x * WP;
-            uint8_t *prx = pre + x * WP;
-            const int X = lo + x, qx = X >> 5;
-            const uint32_t hb = (X & 31) == 31 ? 0u : (FULL << ((X & 31) + 1));
-            int vrun = S.c_vv[x], erun = S.c_e[x];
-            const int e_first = erun;
-            for (int q0 = 0; q0 < W; q0 += 32) {
-                const int qn = min(32, W - q0);
-                uint32_t occ = 0u;
-                for (int u = 0; u < qn; ++u) occ |= (row[q0 + u] != 0u ? 1u : 0u) << u;
-                uint32_t w = 0u, um = 0u;
-                int q = 0;
-                for (;;) {
-                    if (w == 0u) {
-                        if (occ == 0u) break;
-                        q = q0 + __ffs(occ) - 1;
-                        occ &= occ - 1u;
-                        w = row[q];
-                        um = q < qx ? 0u : (q > qx ? FULL : hb);
-                        if (w & um) prx[q] = uint8_t(erun - e_first);
-                        if (q == qx) row[q] = w & hb;
+        tm.sync();
+    }
+
+    // ---------------- B/C2. rows in order: VT sorted, VV read from the bitmaps
+    // A thread sorts two stars of up to 32 tets at once, or one of up to 64:
+    // long chains of register operations on a few warps, while the others
+    // read the VV rows out of the bitmaps.  A sorted entry also gives the
+    // position of its (tet, own vertex) in the row, kept for C3 and C5.
+    {
+        const int half = (nvo + 1) >> 1, nlong = flag[3];
+        const int w_pair = (half + 31) >> 5, w_long = (nlong + 31) >> 5;
+        const int w_emit = do_vv || do_et ? (nvo + 31) >> 5 : 0;
+        for (int w = warp; w < w_pair + w_long + w_emit; w += NWARP) {
+            if (w < w_pair) {
+                const int xa = w * 32 + lane, xb = xa + half;
+                SortRow a{}, b{};
+                if (xa < half) {
+                    a.out = S.vt_off[xa];
+                    a.n = S.vt_off[xa + 1] - a.out;
+                    a.in = row_at(xa);
+                    if (xb < nvo) {
+                        b.out = S.vt_off[xb];
+                        b.n = S.vt_off[xb + 1] - b.out;
+                        b.in = row_at(xb);
                     }
-                    const uint32_t bit = w & (0u - w);
-                    w ^= bit;
-                    const uint16_t id = uint16_t(q * 32 + __ffs(bit) - 1);
-                    if (do_vv) S.st_v[vrun] = id;
-                    ++vrun;
-                    if (bit & um) {
-                        if (do_et) S.st_w[erun] = id;
-                        ++erun;
+                    if (a.n > 32) a.n = 0;
+                    if (b.n > 32) b.n = 0;
+                }
+                const int top = __reduce_max_sync(FULL, max(a.n, b.n));
+                if (top > 24) sort_rows<32>(fill, S.vt_list, S.jpos, keyed, jp16, a, b);
+                else if (top > 16) sort_rows<24>(fill, S.vt_list, S.jpos, keyed, jp16, a, b);
+                else if (top > 0) sort_rows<16>(fill, S.vt_list, S.jpos, keyed, jp16, a, b);
+            } else if (w < w_pair + w_long) {
+                const int i = (w - w_pair) * 32 + lane;
+                SortRow a{}, b{};
+                if (i < nlong) {
+                    const int x = S.long_rows[i];
+                    a.out = S.vt_off[x];
+                    a.n = S.vt_off[x + 1] - a.out;
+                    a.in = row_at(x);
+                    if (a.n > 64) a.n = 0;
+                    if (a.n) {
+                        b.n = a.n - 32;
+                        b.out = a.out + 32;
+                        b.in = a.in + 32;
+                        a.n = 32;
+                    }
+                }
+                sort_rows<64>(fill, S.vt_list, S.jpos, keyed, jp16, a, b);
+            } else {
+                const int x = (w - w_pair - w_long) * 32 + lane;
+                if (x >= nvo) continue;
+                // one loop step per set bit, words visited through an
+                // occupancy mask with the next one loaded ahead
+                const uint32_t *row = bm + x * WP;
+                uint16_t *o = S.st_v + (S.c_vv[x] & kOffMask);
+                for (int q0 = 0; q0 < W; q0 += 32) {
+                    const int qn = min(32, W - q0);
+                    uint32_t occ = 0u;
+#pragma unroll 4
+                    for (int u = 0; u < qn; ++u) occ |= (row[q0 + u] != 0u ? 1u : 0u) << u;
+                    if (occ == 0u) continue;
+                    const uint32_t *r0 = row + q0 - 1;
+                    int f = __ffs(int(occ)), base = 32 * (q0 + f) - 33;
+                    uint32_t wd = r0[f];
+                    occ &= occ - 1u;
+                    f = __ffs(int(occ));
+                    uint32_t next = occ ? r0[f] : 0u;
+                    while (wd) {
+                        *o++ = uint16_t(base + __ffs(int(wd)));
+                        wd &= wd - 1u;
+                        if (wd == 0u) {
+                            wd = next;
+                            base = 32 * (q0 + f) - 33;
+                            occ &= occ - 1u;
+                            f = __ffs(int(occ));
+                            next = occ ? r0[f] : 0u;
+                        }
                     }
                 }
             }
-            bad |= erun - e_first > 255;
         }
-        if (tm.sync_or(bad)) {
-            if (tid == 0) atomicOr(err, ERR_CAPACITY);
-            return true;
+        // stars of more than 64 tets: a warp each
+        if (caps.max_deg > 64)
+            for (int i = warp; i < nlong; i += NWARP) {
+                const int x = S.long_rows[i];
+                const int o = S.vt_off[x], n = S.vt_off[x + 1] - o;
+                if (n <= 64) continue;
+                uint16_t *const v = fill + row_at(x);
+                sort_row_warp(v, n, lane);
+                for (int j = lane; j < n; j += 32) {
+                    const uint32_t e = v[j];
+                    S.vt_list[o + j] = uint16_t(keyed ? e >> 2 : e);
+                    if (keyed && jp16) reinterpret_cast<uint16_t *>(S.jpos)[e] = uint16_t(j);
+                    else if (keyed) S.jpos[e] = uint8_t(j);
+                }
+            }
+        tm.sync();
+        if (!keyed) {  // tet ids too large to carry the slot: positions by a pass over the rows
+            for (int x = warp; x < nvo; x += NWARP) {
+                const int o = S.vt_off[x], n = S.vt_off[x + 1] - o;
+                for (int j = lane; j < n; j += 32) {
+                    const int t = S.vt_list[o + j];
+                    const uint2 r = rows[t];
+                    const uint32_t X = uint32_t(lo + x);
+                    const int s = vtx(r, 0) == X ? 0 : vtx(r, 1) == X ? 1 : vtx(r, 2) == X ? 2 : 3;
+                    if (jp16) reinterpret_cast<uint16_t *>(S.jpos)[4 * t + s] = uint16_t(j);
+                    else S.jpos[4 * t + s] = uint8_t(j);
+                }
+            }
+            tm.sync();
         }
-        if (COUNT && tid == 0) {
-            sizes_out[SZ_VV] = tot[0];
-            sizes_out[SZ_E] = tot[1];
-            sizes_out[SZ_ET] = tot[2];
+    }
+    if (COUNT) {
+        if (tid == 0) {
+            sizes_out[SZ_VT] = vt_total;
+            sizes_out[SZ_VV] = vv_total;
+            sizes_out[SZ_E] = tot_e;
+            sizes_out[SZ_ET] = et_total;
+        }
+    } else {
+        if (mask & R_VT) {
+            for (int i = tid; i <= nvo; i += NT) it->vt_off[i] = S.vt_off[i] + b_vt;
+            copy_out(tm, it->vt_val, vt_total, [&](int j) { return gstar(S.vt_list[j]); });
         }
         if (do_vv) {
-            for (int i = tid; i <= nvo; i += NT) it->vv_off[i] = S.c_vv[i] + b_vv;
-            copy_out(tm, it->vv_val, tot[0], [&](int j) { return vmap[S.st_v[j]]; });
+            for (int i = tid; i <= nvo; i += NT) it->vv_off[i] = (S.c_vv[i] & kOffMask) + b_vv;
+            copy_out(tm, it->vv_val, vv_total, [&](int j) { return vmap[S.st_v[j]]; });
         }
         if (do_et) {
             for (int i = tid; i <= nvo; i += NT) it->eu_off[i] = S.c_e[i] + b_e;
-            copy_out(tm, it->e_w, tot[1], [&](int e) { return vmap[S.st_w[e]]; });
-            if (tid == 0) it->et_off[tot[1]] = tot[2] + b_et;
+            // upper endpoints: the tail of each VV row
+            for (int x = tid; x < nvo; x += NT) {
+                const int e0 = S.c_e[x], ne = S.c_e[x + 1] - e0;
+                const uint16_t *src = S.st_v + (S.c_vv[x + 1] & kOffMask) - ne;
+                int32_t *dst = it->e_w + e0;
+                for (int i = 0; i < ne; ++i) dst[i] = vmap[src[i]];
+            }
+            if (tid == 0) it->et_off[tot_e] = et_total + b_et;
         }
     }
-    if (!(do_et || want_tt)) return true;
-    const int tot_e = tot[1], tot_etv = tot[2];
+    if (!(do_et || want_tt)) {
+        tm.sync();
+        return true;
+    }
     const int nch = plan.nch;
     uint32_t *em = S.emask;
-    tm.sync();  // VV and endpoint staging are dead: r2 takes the edge masks
+    tm.sync();  // the VV staging and the vertex map are dead
+    // the first ET entries move from r2 to the vertex map (nvo <= nv_loc
+    // words), and the edge bases take the place of the VV offsets
+    int32_t *const et_first = S.blk + kHdrWords;
+    for (int x = tid; x < nvo; x += NT) {
+        et_first[x] = et_b[x];
+        cnt[x] = S.c_e[x] - int(uint32_t(cnt[x]) >> 24);
+    }
+    tm.sync();  // r2 takes the edge masks
     fill_words(tm, em, tot_e * nch, 0u);
     tm.sync();
 
     // ---------------- C3. edge tet masks, per tet ----------------
     // bit j of mask(x, w): the j-th tet of VT(x) contains w; every own
-    // vertex x of a tet marks the edges to the tet's vertices above x
+    // vertex x of a tet marks the edges to the tet's vertices above x.  An
+    // internal tet's edge ranks stay in its link words for C5.
     {
-        auto mark = [&](uint32_t x, uint32_t y, uint32_t j) {
-            const int q = int(y >> 5);
-            const int e = S.c_e[x] + int(pre[x * WP + q]) + __popc(bm[x * WP + q] & ((1u << (y & 31)) - 1u));
-            atomicOr(em + e * nch + (j >> 5), 1u << (j & 31));
+        auto rank = [&](uint32_t x, uint32_t y) -> uint32_t {
+            const uint32_t at = x * uint32_t(WP) + (y >> 5);
+            return (pre[at] + uint32_t(__popc(bm[at] & ((1u << (y & 31u)) - 1u)))) & 0xffu;
         };
-        for (int i = tid; i < n_vtets; i += NT) {
-            const uint2 r = rows[i];
-            const uint32_t v0 = r.x & 0xffffu, v1 = r.x >> 16, v2 = r.y & 0xffffu, v3 = r.y >> 16;
-            uint32_t j0, j1, j2;
-            if (jp16) {
-                const uint2 jw = reinterpret_cast<const uint2 *>(S.jpos)[i];
-                j0 = jw.x & 0xffffu;
-                j1 = jw.x >> 16;
-                j2 = jw.y & 0xffffu;
-            } else {
-                const uint32_t jw = reinterpret_cast<const uint32_t *>(S.jpos)[i];
-                j0 = jw & 0xffu;
-                j1 = (jw >> 8) & 0xffu;
-                j2 = (jw >> 16) & 0xffu;
+        auto marks = [&](auto one) {
+            constexpr bool ONE = decltype(one)::value != 0;  // masks of one word
+            auto mark = [&](int e, uint32_t j) {
+                if (ONE) atomicOr(em + e, 1u << j);
+                else atomicOr(em + e * nch + (j >> 5), 1u << (j & 31));
+            };
+            for (int i = tid; i < n_vtets; i += NT) {
+                const uint2 r = rows[i];
+                const uint32_t v0 = r.x & 0xffffu, v1 = r.x >> 16, v2 = r.y & 0xffffu, v3 = r.y >> 16;
+                uint32_t j0, j1, j2;
+                if (!ONE && jp16) {
+                    const uint2 jw = reinterpret_cast<const uint2 *>(S.jpos)[i];
+                    j0 = jw.x & 0xffffu;
+                    j1 = jw.x >> 16;
+                    j2 = jw.y & 0xffffu;
+                } else {
+                    const uint32_t jw = reinterpret_cast<const uint32_t *>(S.jpos)[i];
+                    j0 = jw & 0xffu;
+                    j1 = (jw >> 8) & 0xffu;
+                    j2 = (jw >> 16) & 0xffu;
+                }
+                const uint32_t x0 = v0 - uint32_t(lo), x1 = v1 - uint32_t(lo), x2 = v2 - uint32_t(lo);
+                uint32_t ra = 0u, rb = 0u;
+                if (x0 < nvo_u) {
+                    const int base = cnt[x0];
+                    const uint32_t a = rank(x0, v1), b = rank(x0, v2), c = rank(x0, v3);
+                    mark(base + int(a), j0);
+                    mark(base + int(b), j0);
+                    mark(base + int(c), j0);
+                    ra = a | (b << 8) | (c << 16);
+                }
+                if (x1 < nvo_u) {
+                    const int base = cnt[x1];
+                    const uint32_t a = rank(x1, v2), b = rank(x1, v3);
+                    mark(base + int(a), j1);
+                    mark(base + int(b), j1);
+                    rb = a | (b << 8);
+                }
+                if (x2 < nvo_u) mark(cnt[x2] + int(rank(x2, v3)), j2);
+                if (want_tt && i >= n_ext) reinterpret_cast<uint2 *>(S.nbr)[i - n_ext] = make_uint2(ra, rb);
             }
-            const uint32_t x0 = v0 - uint32_t(lo), x1 = v1 - uint32_t(lo), x2 = v2 - uint32_t(lo);
-            if (x0 < nvo_u) {
-                mark(x0, v1, j0);
-                mark(x0, v2, j0);
-                mark(x0, v3, j0);
-            }
-            if (x1 < nvo_u) {
-                mark(x1, v2, j1);
-                mark(x1, v3, j1);
-            }
-            if (x2 < nvo_u) mark(x2, v3, j2);
-        }
+        };
+        if (nch == 1) marks(IntC<1>{});
+        else marks(IntC<0>{});
     }
     tm.sync();
 
     // ---------------- C5. TT links of faces with an own lowest vertex ------
+    // mask(x, w1) & mask(x, w2), less the tet's own bit, is its partner
+    // across the face (x, w1, w2)
     if (want_tt) {
-        int32_t flags = 0;
-        for (int i = tid; i < n_own; i += NT) {
-            const int li = n_ext + i;
-            const uint2 r = rows[li];
-            const uint32_t v0 = r.x & 0xffffu, v1 = r.x >> 16, v2 = r.y & 0xffffu, v3 = r.y >> 16;
-            const uint32_t a = v0 - uint32_t(lo);
-            if (a >= nvo_u) {  // an internal tet's lowest vertex is own (a part's: an earlier part's)
-                if (!part) flags |= ERR_BAD_BLOCK;
-                continue;
-            }
-            auto rank = [&](uint32_t x, uint32_t y) -> int {
-                const int q = int(y >> 5);
-                return S.c_e[x] + int(pre[x * WP + q]) + __popc(bm[x * WP + q] & ((1u << (y & 31)) - 1u));
-            };
-            // partner of tet li across the face (x, w1, w2): the set bit of
-            // mask(x, w1) & mask(x, w2) other than li's own position js in VT(x)
-            auto link = [&](int e1, int e2, int base, int js, int opp) {
-                const int cs = js >> 5;
-                const uint32_t sb = 1u << (js & 31);
-                int found = 0, partner = -1;
-                for (int c = 0; c < nch; ++c) {
-                    uint32_t mm = em[e1 * nch + c] & em[e2 * nch + c];
-                    if (c == cs) mm &= ~sb;
-                    found += __popc(mm);
-                    if (mm != 0u && partner < 0) partner = S.vt_list[base + c * 32 + __ffs(mm) - 1];
+        auto links = [&](auto one) {
+            constexpr bool ONE = decltype(one)::value != 0;
+            for (int i = tid; i < n_own; i += NT) {
+                const int li = n_ext + i;
+                const uint32_t rx = rows[li].x;
+                const uint2 rk = reinterpret_cast<const uint2 *>(S.nbr)[i];
+                const uint32_t a = (rx & 0xffffu) - uint32_t(lo), b = (rx >> 16) - uint32_t(lo);
+                uint32_t f0 = 0xffffu, f1 = 0xffffu, f2 = 0xffffu, f3 = 0xffffu;
+                auto pick = [&](uint32_t m1, uint32_t m2, uint32_t self, int base, uint32_t &f, int &found) {
+                    const uint32_t mm = m1 & m2 & ~self;
+                    if (mm != 0u) {
+                        if (found == 0) f = S.vt_list[base + __ffs(int(mm)) - 1];
+                        found += ONE ? 1 + ((mm & (mm - 1u)) != 0u) : __popc(mm);
+                    }
+                };
+                if (a < nvo_u) {
+                    const int e = cnt[a], e1 = e + int(rk.x & 0xffu), e2 = e + int((rk.x >> 8) & 0xffu),
+                              e3 = e + int((rk.x >> 16) & 0xffu);
+                    const int base = S.vt_off[a];
+                    int n1 = 0, n2 = 0, n3 = 0;
+                    if (ONE) {
+                        const uint32_t self = 1u << S.jpos[4 * li];
+                        const uint32_t m1 = em[e1], m2 = em[e2], m3 = em[e3];
+                        pick(m1, m2, self, base, f3, n3);
+                        pick(m1, m3, self, base, f2, n2);
+                        pick(m2, m3, self, base, f1, n1);
+                    } else {
+                        const int js = jp16 ? reinterpret_cast<const uint16_t *>(S.jpos)[4 * li] : S.jpos[4 * li];
+                        for (int c = 0; c < nch; ++c) {
+                            const uint32_t self = c == (js >> 5) ? 1u << (js & 31) : 0u;
+                            const uint32_t m1 = em[e1 * nch + c], m2 = em[e2 * nch + c], m3 = em[e3 * nch + c];
+                            pick(m1, m2, self, base + 32 * c, f3, n3);
+                            pick(m1, m3, self, base + 32 * c, f2, n2);
+                            pick(m2, m3, self, base + 32 * c, f1, n1);
+                        }
+                    }
+                    if (max(n1, max(n2, n3)) > 1) flags |= ERR_NONMANIFOLD;
+                    if (b < nvo_u) {
+                        const int eb = cnt[b], e4 = eb + int(rk.y & 0xffu), e5 = eb + int((rk.y >> 8) & 0xffu);
+                        const int base_b = S.vt_off[b];
+                        int n0 = 0;
+                        if (ONE) {
+                            pick(em[e4], em[e5], 1u << S.jpos[4 * li + 1], base_b, f0, n0);
+                        } else {
+                            const int js =
+                                jp16 ? reinterpret_cast<const uint16_t *>(S.jpos)[4 * li + 1] : S.jpos[4 * li + 1];
+                            for (int c = 0; c < nch; ++c)
+                                pick(em[e4 * nch + c], em[e5 * nch + c], c == (js >> 5) ? 1u << (js & 31) : 0u,
+                                     base_b + 32 * c, f0, n0);
+                        }
+                        if (n0 > 1) flags |= ERR_NONMANIFOLD;
+                    }
+                } else if (!part) {  // an internal tet's lowest vertex is own (a part's: an earlier part's)
+                    flags |= ERR_BAD_BLOCK;
                 }
-                if (found > 1) flags |= ERR_NONMANIFOLD;
-                if (partner >= 0) S.nbr[i * 4 + opp] = uint16_t(partner);
-            };
-            const int e1 = rank(a, v1), e2 = rank(a, v2), e3 = rank(a, v3);
-            const int ja = jp16 ? reinterpret_cast<const uint16_t *>(S.jpos)[4 * li] : S.jpos[4 * li];
-            const int jb = jp16 ? reinterpret_cast<const uint16_t *>(S.jpos)[4 * li + 1] : S.jpos[4 * li + 1];
-            const int base_a = S.vt_off[a];
-            link(e1, e2, base_a, ja, 3);
-            link(e1, e3, base_a, ja, 2);
-            link(e2, e3, base_a, ja, 1);
-            const uint32_t b = v1 - uint32_t(lo);
-            if (b < nvo_u) link(rank(b, v2), rank(b, v3), S.vt_off[b], jb, 0);
-        }
+                reinterpret_cast<uint2 *>(S.nbr)[i] = make_uint2(f0 | (f1 << 16), f2 | (f3 << 16));
+            }
+        };
+        if (nch == 1) links(IntC<1>{});
+        else links(IntC<0>{});
         if (GEN && !PART && (flags & ERR_NONMANIFOLD)) {  // TT of this cluster takes the general pass (E')
             flag[2] = 1;
             flags &= ~ERR_NONMANIFOLD;
         }
         if (flags) atomicOr(err, flags);
     }
-    tm.sync();  // bitmaps and rank prefixes are dead: r1 takes the ET staging
+    tm.sync();  // positions, bitmaps and prefixes are dead
 
     // ---------------- C4. ET rows, per edge ----------------
     if (do_et) {
-        uint16_t *st_et = S.st_et;
-        const int per = range_len(tm, tot_e);
-        const int e0 = min(tot_e, tid * per), e1 = min(tot_e, e0 + per);
-        int cnt = 0;
-        for (int e = e0; e < e1; ++e)
-            for (int c = 0; c < nch; ++c) cnt += __popc(em[e * nch + c]);
-        int total;
-        int run = block_scan_thread(tm, cnt, S.scan, &total);
-        if (total != tot_etv) {  // every (own vertex, tet, upper vertex) sets one distinct bit
-            if (tid == 0) atomicOr(err, ERR_BAD_BLOCK);
-            tm.sync();
-            return true;
-        }
-        // own vertex holding edge e0: the largest x with c_e[x] <= e0
-        int xe = 0;
-        if (e0 < e1) {
-            int hi = nvo - 1;
-            while (xe < hi) {
-                const int mid = (xe + hi + 1) >> 1;
-                if (S.c_e[mid] <= e0) xe = mid;
-                else hi = mid - 1;
+        int32_t *eo = S.eo;
+        uint16_t *ex = S.ex;
+        bool bad = false;
+        auto rows_out = [&](auto one) {
+            constexpr bool ONE = decltype(one)::value != 0;
+            const int nc = ONE ? 1 : nch;
+            // each edge's first entry and its lower vertex, per own vertex
+            for (int x = tid; x < nvo; x += NT) {
+                int run = et_first[x];
+                const int e1 = S.c_e[x + 1];
+                for (int e = S.c_e[x]; e < e1; ++e) {
+                    eo[e] = run;
+                    ex[e] = uint16_t(x);
+                    for (int c = 0; c < nc; ++c) run += __popc(em[e * nc + c]);
+                }
+                bad |= run != (x + 1 < nvo ? et_first[x + 1] : et_total);  // one distinct bit per entry
             }
-        }
-        for (int e = e0; e < e1; ++e) {
-            while (S.c_e[xe + 1] <= e) ++xe;
-            const int base = S.vt_off[xe];
-            const int t0 = run;
-            for (int c = 0; c < nch; ++c) {
-                uint32_t mm = em[e * nch + c];
-                while (mm) {
-                    const int b = __ffs(mm) - 1;
-                    mm &= mm - 1;
-                    st_et[run++] = S.vt_list[base + c * 32 + b];
+            bad = tm.sync_or(bad) != 0;
+            if (bad) return;
+            for (int e = tid; e < tot_e; e += NT) {
+                const int o = eo[e];
+                it->et_off[e] = o + b_et;
+                uint16_t *dst = S.st_et + o;
+                const uint16_t *vt = S.vt_list + S.vt_off[ex[e]] - 1;
+                for (int c = 0; c < nc; ++c) {
+                    for (uint32_t mm = em[e * nc + c]; mm; mm &= mm - 1u) *dst++ = vt[__ffs(int(mm))];
+                    vt += 32;
                 }
             }
-            em[e * nch] = uint32_t(t0);  // the edge's first mask word now holds its row offset
+        };
+        if (nch == 1) rows_out(IntC<1>{});
+        else rows_out(IntC<0>{});
+        if (bad) {
+            if (tid == 0) atomicOr(err, ERR_BAD_BLOCK);
+            return true;
         }
         tm.sync();
-        for (int e = tid; e < tot_e; e += NT) it->et_off[e] = int32_t(em[e * nch]) + b_et;
-        copy_out(tm, it->et_val, tot_etv, [&](int j) { return gtet(st_et[j]); });
+        copy_out(tm, it->et_val, et_total, [&](int j) { return gstar(S.st_et[j]); });
         tm.sync();  // ET staging is dead: r1 takes the face hash
     }
 
@@ -918,23 +1138,29 @@ __device__ bool run_cluster(const Team &tm, const DevMesh &m, const SmemPlan &pl
         fill_words(tm, hash, caps.hcap, 0u);
         tm.sync();
         int32_t flags = 0;
+        // the face (b, c, d) an entry stands for: entries hold an internal
+        // tet's index + 1 and, on top, the number of tets matched to its face
+        auto same = [&](uint32_t e, uint2 key) {
+            const uint2 r = rows[n_ext + int(e & kRefMask) - 1];
+            return (r.x >> 16) == key.x && r.y == key.y;
+        };
         // the internal tets whose face (b, c, d) has no own vertex
         const uint16_t *bnd =
             reinterpret_cast<const uint16_t *>(S.blk + blk_bnd_off(h.nv_loc, n_ext, n_own, h.n_halo, xmap));
         for (int jb = tid; jb < h.n_bnd; jb += NT) {
             const int i = bnd[jb];
             const uint2 r = rows[n_ext + i];
-            const uint64_t key = face_key(r, 0);
-            uint32_t hp = face_hash(key, hmask);
+            const uint2 key = make_uint2(r.x >> 16, r.y);
+            uint32_t hp = face_hash(key) & hmask;
             int probe = 0;
             for (; probe < caps.hcap; ++probe) {
-                const uint32_t prev = atomicCAS(&hash[hp], 0u, uint32_t(i * 4 + 1));
+                const uint32_t prev = atomicCAS(&hash[hp], 0u, uint32_t(i + 1));
                 if (prev == 0u) break;
-                const uint32_t ref = (prev & kRefMask) - 1u;
-                if (face_key(rows[n_ext + (ref >> 2)], 0) == key) {
+                if (same(prev, key)) {
+                    const int ref = int(prev & kRefMask) - 1;
                     if (atomicAdd(&hash[hp], kMatch) >= kMatch) flags |= ERR_NONMANIFOLD;
-                    S.nbr[ref] = uint16_t(n_ext + i);
-                    S.nbr[i * 4] = uint16_t(n_ext + (ref >> 2));
+                    S.nbr[4 * ref] = uint16_t(n_ext + i);
+                    S.nbr[4 * i] = uint16_t(n_ext + ref);
                     break;
                 }
                 hp = (hp + 1u) & hmask;
@@ -942,21 +1168,26 @@ __device__ bool run_cluster(const Team &tm, const DevMesh &m, const SmemPlan &pl
             if (probe == caps.hcap) flags |= ERR_HASH_FULL;
         }
         tm.sync();
-        const int n_halo = h.n_halo;
-        for (int j = tid; j < 4 * n_halo; j += NT) {  // one (halo tet, face) per step
-            const int tl = n_vtets + (j >> 2);
-            const uint64_t key = face_key(rows[tl], j & 3);
-            uint32_t hp = face_hash(key, hmask);
-            for (int probe = 0; probe < caps.hcap; ++probe) {
-                const uint32_t e = hash[hp];
-                if (e == 0u) break;
-                const uint32_t ref = (e & kRefMask) - 1u;
-                if (face_key(rows[n_ext + (ref >> 2)], 0) == key) {
-                    if (atomicAdd(&hash[hp], kMatch) >= kMatch) flags |= ERR_NONMANIFOLD;
-                    S.nbr[ref] = uint16_t(tl);
-                    break;
+        for (int j = tid; j < h.n_halo; j += NT) {
+            const int tl = n_vtets + j;
+            const uint2 r = rows[tl];
+#pragma unroll
+            for (int f = 0; f < 4; ++f) {  // the face opposite slot f
+                const uint2 key = f == 0   ? make_uint2(r.x >> 16, r.y)
+                                  : f == 1 ? make_uint2(r.x & 0xffffu, r.y)
+                                  : f == 2 ? make_uint2(r.x & 0xffffu, (r.x >> 16) | (r.y & 0xffff0000u))
+                                           : make_uint2(r.x & 0xffffu, (r.x >> 16) | (r.y << 16));
+                uint32_t hp = face_hash(key) & hmask;
+                for (int probe = 0; probe < caps.hcap; ++probe) {
+                    const uint32_t e = hash[hp];
+                    if (e == 0u) break;
+                    if (same(e, key)) {
+                        if (atomicAdd(&hash[hp], kMatch) >= kMatch) flags |= ERR_NONMANIFOLD;
+                        S.nbr[4 * (int(e & kRefMask) - 1)] = uint16_t(tl);
+                        break;
+                    }
+                    hp = (hp + 1u) & hmask;
                 }
-                hp = (hp + 1u) & hmask;
             }
         }
         if (GEN && !PART && (flags & ERR_NONMANIFOLD)) {
@@ -1566,7 +1797,6 @@ Caps caps_of(const ClusterStat &s, const int64_t *sizes) {
     c.nv_loc = s.nv_loc;
     c.nv_nb = s.nv_nb;
     c.max_deg = s.max_deg;
-    c.max_up = s.max_up;
     c.max_e = s.n_e;
     if (sizes) {
         c.max_vv = int32_t(sizes[SZ_VV]);
@@ -1580,63 +1810,80 @@ Caps caps_of(const ClusterStat &s, const int64_t *sizes) {
     return c;
 }
 
-int64_t estimate_smem(const ClusterStat &s, int threads) {
+int64_t class_bytes(const Caps &c, int threads) {
+    const int64_t nwarp = threads / 32, nvo = c.nv_own;
+    const int64_t W = std::max(1, (c.nv_nb + 31) / 32) | 1, nch = std::max(1, (c.max_deg + 31) / 32);
+    const int64_t pad = (nvo + 1) & ~int64_t(1);
+    const int64_t fixed = 512 + a16(4 * int64_t(c.blk_words)) + 3 * a16(4 * (nvo + 1)) + a16(2 * int64_t(c.n_vt)) +
+                          a16(8 * int64_t(c.n_own)) + a16((c.max_deg > 256 ? 8 : 4) * int64_t(c.n_star));
+    const int64_t edges = a16(std::max<int64_t>(4 * int64_t(c.max_e) * nch,
+                                                a16(2 * int64_t(c.max_vv)) + 2 * int64_t(c.max_e)));
+    const int64_t work = std::max(std::max(a16(2 * nwarp * pad) + 4 * nwarp * pad, a16(4 * nvo * W) + nvo * W),
+                                  std::max(2 * int64_t(c.max_etv), a16(4 * int64_t(c.hcap)) +
+                                                                       a16(4 * (int64_t(c.n_own) + 1)) +
+                                                                       2 * int64_t(c.max_tt)));
+    return fixed + edges + a16(work);
+}
+
+int64_t estimate_class(const ClusterStat &s, int threads) {
     Caps c = caps_of(s, nullptr);
     c.max_vv = 2 * s.n_e;           // each edge is in two VV rows (within the working set, about)
     c.max_etv = s.n_vt + s.n_vt / 2;  // an incidence (x, t) meets 1.5 vertices of t above x on average
     c.max_tt = 4 * s.n_own;
-    return plan_smem(c, threads).total;
+    return class_bytes(c, threads);
 }
 
 SmemPlan plan_smem(const Caps &c, int threads) {
     SmemPlan p{};
     p.threads = threads;
     p.caps = c;
-    const int64_t nwarp = threads / 32;
     const int64_t nvo = c.nv_own;
     p.W = std::max(1, (c.nv_nb + 31) / 32) | 1;  // row stride of the bitmaps (odd)
     p.nch = std::max(1, (c.max_deg + 31) / 32);
-    p.pad = int32_t((nvo + 1) & ~int64_t(1));
-    int64_t off = 0;
-    p.scan = 0;
-    off = a16(4 * 128);
-    p.blk = int32_t(off);
-    off = a16(off + 4 * int64_t(c.blk_words));
-    p.vt_off = int32_t(off);
-    off = a16(off + 4 * (nvo + 1));
-    p.vt_list = int32_t(off);
-    off = a16(off + 2 * int64_t(c.n_vt));
-    p.c_vv = int32_t(off);
-    off = a16(off + 4 * (nvo + 1));
-    p.c_e = int32_t(off);
-    off = a16(off + 4 * (nvo + 1));
-    p.nbr = int32_t(off);
-    off = a16(off + 8 * int64_t(c.n_own));
-    p.jpos16 = c.max_deg > 256 ? 1 : 0;
-    p.jpos = int32_t(off);
-    off = a16(off + (p.jpos16 ? 8 : 4) * int64_t(c.n_star));
-    // r2: VV staging + upper-endpoint staging, then the edge masks
-    p.r2 = int32_t(off);
-    p.st_w = int32_t(a16(off + 2 * int64_t(c.max_vv)));
-    const int64_t r2 = std::max<int64_t>(4 * int64_t(c.max_e) * p.nch,
-                                         a16(2 * int64_t(c.max_vv)) + 2 * int64_t(c.max_e));
-    off = a16(off + r2);
-    // r1: phase B counters + lane masks | bitmaps + rank prefixes | ET
-    // staging | face hash + TT counts + TT staging
-    p.r1 = int32_t(off);
-    const int64_t cw = a16(2 * nwarp * p.pad);
-    p.mk = int32_t(off + cw);
-    const int64_t bm = a16(4 * nvo * p.W);
-    p.pre = int32_t(off + bm);
-    const int64_t hs = a16(4 * int64_t(c.hcap));
-    p.tcnt = int32_t(off + hs);
-    const int64_t tc = a16(4 * (int64_t(c.n_own) + 1));
-    p.st_tt = int32_t(off + hs + tc);
-    const int64_t r1 = std::max(std::max(cw + 4 * nwarp * p.pad, bm + nvo * p.W),
-                                std::max(2 * int64_t(c.max_etv), hs + tc + 2 * int64_t(c.max_tt)));
-    off = a16(off + r1);
-    p.total = off > INT32_MAX ? INT32_MAX : int32_t(off);
-    return p;
+    p.mode = (c.max_deg > 256 ? kJpos16 : 0) | (c.n_star <= 16383 ? kKeyed : 0);  // 4 * tet + slot below 0xffff
+    // The fill's rows are padded to one odd number of words (no count pass
+    // before it, and a thread per row meets no bank conflict) unless that
+    // takes over a quarter more than compact rows, as on irregular meshes.
+    const int64_t stride = 2 * (((c.max_deg + 1) / 2) | 1);
+    p.stride = c.max_deg <= 62 && 4 * nvo * stride <= 5 * int64_t(c.n_vt) ? int32_t(stride) : 0;
+    for (;;) {
+        int64_t off = 0;
+        auto take = [&](int64_t bytes) {
+            const int64_t at = off;
+            off = a16(off + bytes);
+            return int32_t(std::min<int64_t>(at, INT32_MAX));
+        };
+        p.scan = take(4 * scan_words(threads));
+        p.blk = take(4 * int64_t(c.blk_words));
+        p.vt_off = take(4 * (nvo + 1));
+        p.vt_list = take(2 * int64_t(c.n_vt));
+        p.c_vv = take(4 * (nvo + 1));
+        p.c_e = take(4 * (nvo + 1));
+        p.jpos = take(std::max((p.mode & kJpos16 ? 8 : 4) * int64_t(c.n_star), 4 * int64_t(c.max_e)));
+        // r2: fill cursors, then VV staging; first ET entries, long rows; then
+        // the edge masks.  The rows in arrival order (padded, or compact from a
+        // word each) end with nbr and reach back into what r2 leaves free.
+        const int64_t vv = a16(std::max(2 * int64_t(c.max_vv), 4 * nvo)), eb = a16(4 * nvo);
+        const int64_t lr = c.max_deg > 32 ? a16(2 * nvo) : 0;
+        p.r2 = take(std::max<int64_t>(4 * int64_t(c.max_e) * p.nch, vv + eb + lr));
+        p.et_b = int32_t(p.r2 + vv);
+        p.long_rows = int32_t(p.r2 + vv + eb);
+        const int64_t n_fill = a16(p.stride ? 2 * nvo * p.stride : 2 * (int64_t(c.n_vt) + nvo + 4));
+        p.nbr = take(std::max(8 * int64_t(c.n_own), p.r2 + vv + eb + lr + n_fill - off));
+        p.fill = int32_t(std::min<int64_t>(off - n_fill, INT32_MAX));
+        // r1: bitmaps + rank prefixes | ET staging + the edges' lower vertices
+        // | face hash + TT counts + TT staging
+        const int64_t bm = a16(4 * nvo * p.W), et = a16(2 * int64_t(c.max_etv));
+        const int64_t hs = a16(4 * int64_t(c.hcap)), tc = a16(4 * (int64_t(c.n_own) + 1));
+        p.r1 = take(std::max(std::max(bm + nvo * p.W, et + 2 * int64_t(c.max_e)), hs + tc + 2 * int64_t(c.max_tt)));
+        p.pre = int32_t(p.r1 + bm);
+        p.ex = int32_t(p.r1 + et);
+        p.tcnt = int32_t(p.r1 + hs);
+        p.st_tt = int32_t(p.r1 + hs + tc);
+        p.total = off > INT32_MAX ? INT32_MAX : int32_t(off);
+        if (!p.stride || off <= kPaddedFit) return p;
+        p.stride = 0;  // compact rows take less
+    }
 }
 
 int kernel_smem_limit() {

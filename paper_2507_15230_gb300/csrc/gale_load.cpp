@@ -554,7 +554,7 @@ bool prepare_host(const gale_mesh_desc &d, HostMesh &hm, std::string &err) {
     std::vector<int32_t> cutk;
     for (int32_t k = 0; k < K; ++k) {
         const ClusterStat &s = hm.stats[k];
-        if (d.part_vertices >= 0 && s.nv_own >= 2 && estimate_smem(s, 512) > cut_bytes) cutk.push_back(k);
+        if (d.part_vertices >= 0 && s.nv_own >= 2 && estimate_class(s, 512) > cut_bytes) cutk.push_back(k);
     }
     struct PartBuild {
         int32_t a0 = 0, a1 = 0, n_rows = 0;
@@ -630,7 +630,7 @@ bool prepare_host(const gale_mesh_desc &d, HostMesh &hm, std::string &err) {
                     bad_p = k;
                     return;
                 }
-                fit &= estimate_smem(pbs[j].s, 512) <= kPartFitBytes;
+                fit &= estimate_class(pbs[j].s, 512) <= kPartFitBytes;
             }
             if (fit || S >= nvo) break;
             S = std::min(nvo, 2 * S);
