@@ -81,6 +81,8 @@ int threads_for(const gale_ctx *ctx, const gale::ClusterStat &s) {
     return t;
 }
 
+constexpr int kMergedThreads = 512;
+
 // Size bins: work items (clusters, then the parts of cut clusters) sorted by
 // shared-memory need, cut where the merged plan would cross the next
 // occupancy tier (4, 3, 2, 1 CTAs per SM).  Items whose plan exceeds the
@@ -98,6 +100,12 @@ gale_status plan_bins(gale_ctx *ctx, bool with_sizes) {
     const int smem_cta = gale::dynamic_smem_limit();
     int smem_sm = 0;
     cudaDeviceGetAttribute(&smem_sm, cudaDevAttrMaxSharedMemoryPerMultiprocessor, ctx->device);
+    ctx->smem_sm = smem_sm;
+    {
+        gale::SmemPlan p{};
+        p.threads = kMergedThreads;
+        ctx->merged_per_sm = gale::max_ctas_per_sm(p, false, true);
+    }
     auto caps_k = [&](int32_t k) {
         return gale::caps_of(ctx->hm.stats[k], with_sizes ? ctx->sizes.data() + size_t(5) * k : nullptr);
     };
@@ -181,6 +189,8 @@ gale_status plan_bins(gale_ctx *ctx, bool with_sizes) {
     // keep their own plan (one persistent launch, the largest member's
     // shared memory).
     ctx->h_plans.assign(size_t(NI), gale::SmemPlan{});
+    if (with_sizes)
+        for (int32_t k = 0; k < NI; ++k) ctx->h_plans[k] = gale::plan_smem(caps_k(k), thr[k]);
     {
         // (block size, bin of cut clusters) -> bins of the top tier
         using Key = std::pair<int, bool>;
@@ -324,6 +334,37 @@ SmemPlan serve_plan(gale_ctx *ctx, bool *fits, std::vector<uint8_t> *in_loop, st
     if (in_loop) *in_loop = sel;
     return env;
 }
+// Short lists.  Size bins are launched one after another or side by side,
+// each with its own block size and occupancy, which pays when a bin fills the
+// GPU.  Where every listed item has a CTA's place at once, one launch of
+// kMergedThreads-thread CTAs, each under its item's own plan, is faster: it
+// takes the longest item's time, not the sum over the bins of each bin's, and
+// more threads an item than the bins' rule gives small ones.  Measured: 16^3
+// grid (two bins of 64 and 128 threads) 73.8 us alone, as one bin of 512
+// threads 41.4; 3 clusters of a Delaunay mesh in three bins 151 us.  The line
+// lies where the items no longer all fit.  A block size or occupancy set by
+// the caller, teams and global-scratch bins keep their bins' launches.
+bool merged_launch(const gale_ctx *ctx, const int32_t *items, int32_t n, SmemPlan *env) {
+    if (n < 1 || ctx->threads_override || ctx->ctas_override || n > ctx->merged_per_sm * ctx->sm_count) return false;
+    int top = 0, first = -1;
+    bool several = false;
+    for (int32_t i = 0; i < n; ++i) {
+        const int32_t b = ctx->bin_of[items[i]];
+        if (b < 0) return false;
+        const Bin &bin = ctx->bins[b];
+        if (bin.spill || bin.teams > 0) return false;
+        several |= (first >= 0 && b != first) || bin.plan.threads < kMergedThreads;
+        first = b;
+        top = std::max(top, ctx->h_plans[items[i]].total);
+    }
+    const int per_sm = std::min(ctx->merged_per_sm, ctx->smem_sm / (top + 1024 + 512));
+    if (!several || n > per_sm * ctx->sm_count) return false;
+    *env = SmemPlan{};
+    env->threads = kMergedThreads;
+    env->total = top;
+    return true;
+}
+
 // Lengths of the ten output arrays of cluster k under mask.
 void item_lengths(const gale_ctx *ctx, int32_t k, uint32_t mask, int64_t *L) {
     const int64_t *sz = ctx->sizes.data() + size_t(5) * k;
@@ -537,6 +578,73 @@ bool chunk_bin_orders(const gale_ctx *ctx, const std::vector<int32_t> &list, boo
     return run == cnt;
 }
 
+// One size bin's share of a batched build: n items, order[] into `items`.
+struct BinRun {
+    size_t bin;
+    const int32_t *order;
+    int32_t n;
+};
+
+constexpr int kBinStreams = 5;  // beside the context's own
+
+cudaError_t ensure_bin_streams(gale_ctx *ctx, size_t ns) {
+    while (ctx->bin_streams.size() < ns) {
+        cudaStream_t st;
+        const cudaError_t e = cudaStreamCreateWithFlags(&st, cudaStreamNonBlocking);
+        if (e != cudaSuccess) return e;
+        ctx->bin_streams.push_back(st);
+    }
+    while (ctx->bin_events.size() < ns + 1) {
+        cudaEvent_t ev;
+        const cudaError_t e = cudaEventCreateWithFlags(&ev, cudaEventDisableTiming);
+        if (e != cudaSuccess) return e;
+        ctx->bin_events.push_back(ev);
+    }
+    return cudaSuccess;
+}
+
+// The bins' launches, after the placement pass on the context stream (which
+// zeroed the tickets).  Several bins run side by side: forked to streams of
+// the context and joined again, so that one bin's last CTAs share the GPU
+// with the next one's (2e5-point Delaunay mesh, six bins of 1,500 items: 459
+// us one after another).  The largest CTAs go first; bins in global
+// scratch share it and stay in one stream.  Works under stream capture.
+cudaError_t run_bins(gale_ctx *ctx, const gale::DevMesh &dm, const WorkItem *items, std::vector<BinRun> runs,
+                     int64_t *launches) {
+    cudaStream_t s = ctx->stream;
+    auto launch = [&](const BinRun &r, cudaStream_t st) {
+        const gale::Bin &bin = ctx->bins[r.bin];
+        ++*launches;
+        return cudaError_t(gale::launch_build(dm, bin.plan, items, r.order, r.n, ctx->d_err, ctx->d_tickets + r.bin,
+                                              grid_of(bin, r.n), st, scratch_of(ctx, bin), plans_of(ctx, bin),
+                                              bin.teams, false));
+    };
+    if (runs.size() <= 1) return runs.empty() ? cudaSuccess : launch(runs[0], s);
+    std::stable_sort(runs.begin(), runs.end(), [&](const BinRun &a, const BinRun &b) {
+        const gale::Bin &x = ctx->bins[a.bin], &y = ctx->bins[b.bin];
+        if (x.spill != y.spill) return x.spill > y.spill;
+        return x.plan.total > y.plan.total;
+    });
+    const size_t ns = std::min<size_t>(runs.size() - 1, kBinStreams);
+    cudaError_t e = ensure_bin_streams(ctx, ns);
+    if (e == cudaSuccess) e = cudaEventRecord(ctx->bin_events[ns], s);
+    if (e != cudaSuccess) return e;
+    for (size_t i = 0; e == cudaSuccess && i < ns; ++i) e = cudaStreamWaitEvent(ctx->bin_streams[i], ctx->bin_events[ns], 0);
+    size_t next = 0;  // streams in turn; the global-scratch bins, which come first, in the context's
+    for (size_t i = 0; e == cudaSuccess && i < runs.size(); ++i) {
+        const bool own = ctx->bins[runs[i].bin].spill || next % (ns + 1) == ns;
+        e = launch(runs[i], own ? s : ctx->bin_streams[next % (ns + 1)]);
+        if (!ctx->bins[runs[i].bin].spill) ++next;
+    }
+    // joined even after a failed launch: a capture must not end forked
+    for (size_t i = 0; i < ns; ++i) {
+        cudaError_t j = cudaEventRecord(ctx->bin_events[i], ctx->bin_streams[i]);
+        if (j == cudaSuccess) j = cudaStreamWaitEvent(s, ctx->bin_events[i], 0);
+        if (e == cudaSuccess) e = j;
+    }
+    return e;
+}
+
 gale_status ensure_bulk(gale_ctx *ctx, const int64_t *need) {
     bool realloc = false;
     for (int a = 0; a < 10; ++a) {
@@ -734,6 +842,8 @@ void gale_destroy(gale_ctx *ctx) {
             cudaStreamDestroy(ctx->copy_stream);
         }
         for (cudaEvent_t e : ctx->chunk_events) cudaEventDestroy(e);
+        for (cudaEvent_t e : ctx->bin_events) cudaEventDestroy(e);
+        for (cudaStream_t st : ctx->bin_streams) cudaStreamDestroy(st);
         for (int b = 0; b < 2; ++b) {
             if (ctx->stage[b]) cudaFreeHost(ctx->stage[b]);
             if (ctx->stage_ev[b]) cudaEventDestroy(ctx->stage_ev[b]);
@@ -910,18 +1020,29 @@ gale_status gale_build_clusters(gale_ctx *ctx, const int32_t *ids, int32_t n, ui
         cudaGraphExec_t &g = ctx->graphs[mask];
         if (!g) {
             cudaGraph_t graph;
+            const int32_t ni = int32_t(ctx->all_items.size());
+            gale::SmemPlan env;
+            const bool merged = gale::merged_launch(ctx, ctx->all_items.data(), ni, &env);
+            std::vector<BinRun> runs;
+            for (size_t b = 0; !merged && b < ctx->bins.size(); ++b)
+                if (!ctx->bins[b].cut)  // a cut bin's clusters' parts are in other bins
+                    runs.push_back({b, ctx->d_order_all + ctx->order_all_off[b], int32_t(ctx->bins[b].clusters.size())});
+            if (runs.size() > 1)  // not while capturing
+                CUDA_TRY(ensure_bin_streams(ctx, std::min<size_t>(runs.size() - 1, kBinStreams)));
             CUDA_TRY(cudaStreamBeginCapture(ctx->stream, cudaStreamCaptureModeThreadLocal));
-            int rc = gale::launch_bases(dm, ctx->hm.NP ? ctx->d_all_items : nullptr, int32_t(ctx->all_items.size()),
-                                        ctx->d_sizes, mask, base, ctx->d_items, ctx->d_totals, ctx->d_bsum,
-                                        ctx->stream);
-            for (size_t b = 0; rc == 0 && b < ctx->bins.size(); ++b) {
-                const gale::Bin &bin = ctx->bins[b];
-                if (bin.cut) continue;  // its clusters' parts are in other bins
-                rc = gale::launch_build(dm, bin.plan, ctx->d_items, ctx->d_order_all + ctx->order_all_off[b],
-                                        int32_t(bin.clusters.size()), ctx->d_err, ctx->d_tickets + b,
-                                        grid_of(bin, int32_t(bin.clusters.size())), ctx->stream, scratch_of(ctx, bin),
-                                        plans_of(ctx, bin), bin.teams);
+            int nl = 0;
+            int64_t builds = 0;
+            int rc = gale::launch_bases(dm, ctx->hm.NP ? ctx->d_all_items : nullptr, ni, ctx->d_sizes, mask, base,
+                                        ctx->d_items, ctx->d_totals, ctx->d_bsum, ctx->d_tickets,
+                                        int(ctx->bins.size()), ctx->stream, &nl);
+            if (rc == 0 && merged) {
+                builds = 1;
+                rc = gale::launch_build(dm, env, ctx->d_items, nullptr, ni, ctx->d_err, ctx->d_tickets, ni, ctx->stream,
+                                        nullptr, ctx->d_plans, 0, false);
+            } else if (rc == 0) {
+                rc = int(run_bins(ctx, dm, ctx->d_items, std::move(runs), &builds));
             }
+            ctx->graph_launches[mask] = nl + builds;
             cudaError_t ce = cudaStreamEndCapture(ctx->stream, &graph);
             if (rc != 0) return cuda_fail(cudaError_t(rc), "capturing the batched build");
             if (ce != cudaSuccess) return cuda_fail(ce, "cudaStreamEndCapture");
@@ -933,8 +1054,7 @@ gale_status gale_build_clusters(gale_ctx *ctx, const int32_t *ids, int32_t n, ui
             }
         }
         CUDA_TRY(cudaGraphLaunch(g, ctx->stream));
-        launches = 3;
-        for (const auto &bin : ctx->bins) launches += !bin.cut;
+        launches = ctx->graph_launches[mask];
     } else {
         // a partial batched build lists the parts of cut clusters in their place
         const std::vector<int32_t> items = mode == GALE_MODE_BATCHED ? expand_items(ctx, list) : list;
@@ -944,10 +1064,12 @@ gale_status gale_build_clusters(gale_ctx *ctx, const int32_t *ids, int32_t n, ui
             CUDA_TRY(cudaMemcpyAsync(ctx->d_ids, items.data(), size_t(ni) * 4, cudaMemcpyHostToDevice, ctx->stream));
             d_ids = ctx->d_ids;
         }
+        int nl = 0;
         int rc = gale::launch_bases(dm, d_ids, ni, ctx->d_sizes, mask, base, ctx->d_items, ctx->d_totals,
-                                    ctx->d_bsum, ctx->stream);
+                                    ctx->d_bsum, ctx->d_tickets, int(ctx->bins.size()), ctx->stream, &nl);
         if (rc != 0) return cuda_fail(cudaError_t(rc), "bases launch");
-        launches = 3;
+        launches = nl;
+        gale::SmemPlan env;
         if (mode == GALE_MODE_PER_CLUSTER) {
             for (int32_t i = 0; i < cnt; ++i) {
                 const gale::Bin &bin = ctx->bins[ctx->bin_of[list[i]]];
@@ -956,6 +1078,11 @@ gale_status gale_build_clusters(gale_ctx *ctx, const int32_t *ids, int32_t n, ui
                 if (rc != 0) return cuda_fail(cudaError_t(rc), "per-cluster launch");
             }
             launches += cnt;
+        } else if (gale::merged_launch(ctx, items.data(), ni, &env)) {
+            rc = gale::launch_build(dm, env, ctx->d_items, nullptr, ni, ctx->d_err, ctx->d_tickets, ni, ctx->stream,
+                                    nullptr, ctx->d_plans, 0, false);
+            if (rc != 0) return cuda_fail(cudaError_t(rc), "batched launch");
+            ++launches;
         } else {
             // partial batched build: per-bin item orders
             std::vector<int32_t> order;
@@ -965,16 +1092,11 @@ gale_status gale_build_clusters(gale_ctx *ctx, const int32_t *ids, int32_t n, ui
             const std::vector<int64_t> &off = boff[0];
             CUDA_TRY(cudaMemcpyAsync(ctx->d_order_part, order.data(), order.size() * 4, cudaMemcpyHostToDevice,
                                      ctx->stream));
-            for (size_t b = 0; b < ctx->bins.size(); ++b) {
-                const int32_t nb = int32_t(off[b + 1] - off[b]);
-                if (nb == 0) continue;
-                const gale::Bin &bin = ctx->bins[b];
-                rc = gale::launch_build(dm, bin.plan, ctx->d_items, ctx->d_order_part + off[b], nb, ctx->d_err,
-                                        ctx->d_tickets + b, grid_of(bin, nb), ctx->stream, scratch_of(ctx, bin),
-                                        plans_of(ctx, bin), bin.teams);
-                if (rc != 0) return cuda_fail(cudaError_t(rc), "batched launch");
-                ++launches;
-            }
+            std::vector<BinRun> runs;
+            for (size_t b = 0; b < ctx->bins.size(); ++b)
+                if (off[b + 1] > off[b]) runs.push_back({b, ctx->d_order_part + off[b], int32_t(off[b + 1] - off[b])});
+            const cudaError_t re = run_bins(ctx, dm, ctx->d_items, std::move(runs), &launches);
+            if (re != cudaSuccess) return cuda_fail(re, "batched launch");
         }
     }
     ctx->last_launches = launches;
@@ -1161,19 +1283,25 @@ gale_status gale_build_export(gale_ctx *ctx, const int32_t *ids, int32_t n, uint
         const int32_t i0 = cut[c];
         const int32_t j0 = icut[c], nc = icut[c + 1] - j0;
         if (nc > 0) {
+            int nl = 0;
             int rc = gale::launch_bases(dm, ctx->d_ids + j0, nc, ctx->d_sizes, mask, ctx->d_chunk_base + c,
-                                        ctx->d_items + j0, ctx->d_totals, ctx->d_bsum, ctx->stream);
+                                        ctx->d_items + j0, ctx->d_totals, ctx->d_bsum, ctx->d_tickets,
+                                        int(ctx->bins.size()), ctx->stream, &nl);
             if (rc != 0) return cuda_fail(cudaError_t(rc), "bases launch");
-            launches += 3;
-            for (size_t b = 0; b < ctx->bins.size(); ++b) {
-                const int32_t nb = int32_t(boff[c][b + 1] - boff[c][b]);
-                if (nb == 0) continue;
-                const gale::Bin &bin = ctx->bins[b];
-                rc = gale::launch_build(dm, bin.plan, ctx->d_items + j0, ctx->d_order_part + boff[c][b], nb,
-                                        ctx->d_err, ctx->d_tickets + b, grid_of(bin, nb), ctx->stream,
-                                        scratch_of(ctx, bin), plans_of(ctx, bin), bin.teams);
+            launches += nl;
+            gale::SmemPlan env;
+            if (gale::merged_launch(ctx, items.data() + j0, nc, &env)) {
+                rc = gale::launch_build(dm, env, ctx->d_items + j0, nullptr, nc, ctx->d_err, ctx->d_tickets, nc,
+                                        ctx->stream, nullptr, ctx->d_plans, 0, false);
                 if (rc != 0) return cuda_fail(cudaError_t(rc), "batched launch");
                 ++launches;
+            } else {
+                std::vector<BinRun> runs;
+                for (size_t b = 0; b < ctx->bins.size(); ++b)
+                    if (boff[c][b + 1] > boff[c][b])
+                        runs.push_back({b, ctx->d_order_part + boff[c][b], int32_t(boff[c][b + 1] - boff[c][b])});
+                const cudaError_t re = run_bins(ctx, dm, ctx->d_items + j0, std::move(runs), &launches);
+                if (re != cudaSuccess) return cuda_fail(re, "batched launch");
             }
         }
         // the chunk's outputs leave while the next chunk builds
@@ -1362,7 +1490,7 @@ gale_status gale_autotune(gale_ctx *ctx, uint32_t mask, int32_t reps, float *bes
     const gale::DevMesh dm = dev_mesh(ctx);
     int rc = gale::launch_bases(dm, ctx->hm.NP ? ctx->d_all_items : nullptr, int32_t(ctx->all_items.size()),
                                 ctx->d_sizes, mask, ctx->d_arrays_base + mask, ctx->d_items, ctx->d_totals,
-                                ctx->d_bsum, ctx->stream);
+                                ctx->d_bsum, ctx->d_tickets, 0, ctx->stream);
     if (rc != 0) return cuda_fail(cudaError_t(rc), "bases launch");
     const int smem_limit = gale::dynamic_smem_limit();
     if (!gale::prepare_kernels(smem_limit)) return fail(GALE_ECUDA, "setting the kernels' shared memory limit failed");

@@ -76,7 +76,7 @@ struct gale_ctx {
     int64_t *d_totals = nullptr;            // [10]
     int64_t *d_bsum = nullptr;              // output placement scratch
     char *d_spill = nullptr;                // per-CTA regions of spill bins
-    gale::SmemPlan *d_plans = nullptr;      // [K+NP] own plans of the members of per-item bins
+    gale::SmemPlan *d_plans = nullptr;      // [K+NP] every item's own plan (per-item bins, merged launches)
     std::vector<gale::SmemPlan> h_plans;    // host copy
     int64_t spill_bytes = 0;
     std::vector<int64_t> sizes;             // host [(K+NP)*5]
@@ -91,6 +91,8 @@ struct gale_ctx {
     int threads_override = 0;  // 0: chosen from the cluster's tet count
     int ctas_override = 0;
     int sm_count = 0;
+    int smem_sm = 0;        // shared memory of an SM
+    int merged_per_sm = 0;  // CTAs of a merged launch an SM holds by threads and registers
 
     // bulk output arrays
     int32_t *bulk[10] = {};
@@ -99,6 +101,10 @@ struct gale_ctx {
     std::vector<int64_t> bulk_offs;  // [n*10]
     std::vector<int32_t> bulk_ids;
     uint32_t bulk_mask = 0;
+
+    // streams and events that several size bins' launches fork to and join by
+    std::vector<cudaStream_t> bin_streams;
+    std::vector<cudaEvent_t> bin_events;
 
     // pipelined build + export: copy stream, chunk events, chunk base items
     cudaStream_t copy_stream = nullptr;
@@ -113,6 +119,7 @@ struct gale_ctx {
 
     // captured full builds, one per mask
     cudaGraphExec_t graphs[16] = {};
+    int64_t graph_launches[16] = {};
     int64_t last_launches = 0;
 
     std::vector<gale::DevAlloc> allocs;
@@ -138,6 +145,9 @@ namespace gale {
 gale_status copy_to_host(gale_ctx *ctx, void *dst, const void *src, size_t bytes);
 // Lengths of the ten output arrays of cluster k under mask (gale_api.cpp).
 void item_lengths(const gale_ctx *ctx, int32_t k, uint32_t mask, int64_t *L);
+// Whether these work items are built by one merged launch (gale_api.cpp):
+// *env gets its block size and shared memory.
+bool merged_launch(const gale_ctx *ctx, const int32_t *items, int32_t n, SmemPlan *env);
 void enumeration_destroy(gale_ctx *ctx);  // gale_enum.cpp
 void cobound_destroy(gale_ctx *ctx);      // gale_cobound.cu
 }  // namespace gale

@@ -258,17 +258,19 @@ struct DevMesh {
 int launch_count_pass(const DevMesh &m, const SmemPlan &plan, const int32_t *ids, int32_t n, int64_t *sizes_out,
                       int32_t *err, int32_t *ticket, int grid, void *stream, char *gscratch, uint32_t mask,
                       const SmemPlan *plans = nullptr);
-// Output placement for n listed clusters (three launches).  bsum: device
-// scratch of bases_scratch_words(n) int64 words.
+// Output placement for n listed clusters (one launch up to 1,024 of them, else
+// three), which also zeroes the nt (at most 256) ticket counters of the builds
+// that follow.  bsum: device scratch of bases_scratch_words(n) int64 words.
 int bases_scratch_words(int32_t n);
 int launch_bases(const DevMesh &m, const int32_t *ids, int32_t n, const int64_t *sizes, uint32_t mask,
-                 const WorkItem *arrays_base, WorkItem *items, int64_t *totals_out, int64_t *bsum, void *stream);
+                 const WorkItem *arrays_base, WorkItem *items, int64_t *totals_out, int64_t *bsum, int32_t *tickets,
+                 int nt, void *stream, int *launches = nullptr);
 // teams > 0: several clusters per CTA, one team of plan.threads threads each
 // (`teams` of them per CTA, each with plan.total bytes of shared memory);
-// never with plans or gscratch.
+// never with plans or gscratch.  reset: zero the ticket counter first.
 int launch_build(const DevMesh &m, const SmemPlan &plan, const WorkItem *items, const int32_t *order, int32_t n,
                  int32_t *err, int32_t *ticket, int grid, void *stream, char *gscratch,
-                 const SmemPlan *plans = nullptr, int teams = 0);
+                 const SmemPlan *plans = nullptr, int teams = 0, bool reset = true);
 // One launch, one CTA, one work item (the per-cluster baseline form).
 int launch_build_one(const DevMesh &m, const SmemPlan &plan, const WorkItem *items, int32_t index, int32_t *err,
                      void *stream, char *gscratch);

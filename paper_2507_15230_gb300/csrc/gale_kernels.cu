@@ -1637,7 +1637,7 @@ __global__ void __launch_bounds__(1024) serve_kernel(DevMesh m, const SmemPlan *
 // Output placement: exclusive scans, over the listed clusters, of the
 // lengths of the ten output arrays, then one work item per cluster with its
 // output pointers.  Three launches: block sums, a scan of the block sums,
-// then per-block scans that write the items.  arrays_base holds the base
+// then per-block scans that write the items (one launch for short lists).  arrays_base holds the base
 // pointers of the ten output arrays (its k / mask / blk fields are ignored).
 constexpr int kBasesThreads = 256;
 constexpr int NA = 10;
@@ -1709,10 +1709,11 @@ __device__ __forceinline__ void block_scan_na(int64_t *v, int64_t (*s_warp)[NA],
 
 __global__ void __launch_bounds__(kBasesThreads) bases_sum_kernel(DevMesh m, const int32_t *ids, int32_t n,
                                                                   const int64_t *sizes, uint32_t mask,
-                                                                  int64_t *bsum) {
+                                                                  int64_t *bsum, int32_t *tickets, int nt) {
     __shared__ int64_t s_warp[32][NA];
     __shared__ int64_t s_tot[NA];
     const int idx = blockIdx.x * blockDim.x + threadIdx.x;
+    if (blockIdx.x == 0 && int(threadIdx.x) < nt) tickets[threadIdx.x] = 0;
     int64_t L[NA];
     if (idx < n) item_lengths(m, ids, sizes, mask, idx, L);
     else
@@ -1742,6 +1743,23 @@ __global__ void __launch_bounds__(kBasesThreads) bases_scan_kernel(int32_t nbloc
     if (threadIdx.x < NA) totals[threadIdx.x] = s_run[threadIdx.x];
 }
 
+// the idx-th work item: its arrays start `run` after `before` in each base
+__device__ __forceinline__ void write_item(const DevMesh &m, const int32_t *ids, int idx, uint32_t mask,
+                                           int32_t *const *base, const int64_t *before, const int64_t *run,
+                                           WorkItem *items) {
+    const int k = ids ? ids[idx] : idx;
+    WorkItem w;
+    w.k = k;
+    w.mask = mask;
+    w.blk = m.blk_off[k];
+    int32_t *p[NA];
+    for (int a = 0; a < NA; ++a) p[a] = base[a] ? base[a] + before[a] + run[a] : nullptr;
+    w.vt_off = p[0]; w.vt_val = p[1]; w.vv_off = p[2]; w.vv_val = p[3];
+    w.eu_off = p[4]; w.e_w = p[5]; w.et_off = p[6]; w.et_val = p[7];
+    w.tt_off = p[8]; w.tt_val = p[9];
+    items[idx] = w;
+}
+
 __global__ void __launch_bounds__(kBasesThreads) bases_write_kernel(DevMesh m, const int32_t *ids, int32_t n,
                                                                     const int64_t *sizes, uint32_t mask,
                                                                     const WorkItem *arrays_base,
@@ -1761,17 +1779,38 @@ __global__ void __launch_bounds__(kBasesThreads) bases_write_kernel(DevMesh m, c
     int32_t *base[NA] = {arrays_base->vt_off, arrays_base->vt_val, arrays_base->vv_off, arrays_base->vv_val,
                          arrays_base->eu_off, arrays_base->e_w,    arrays_base->et_off, arrays_base->et_val,
                          arrays_base->tt_off, arrays_base->tt_val};
-    const int k = ids ? ids[idx] : idx;
-    WorkItem w;
-    w.k = k;
-    w.mask = mask;
-    w.blk = m.blk_off[k];
-    int32_t *p[NA];
-    for (int a = 0; a < NA; ++a) p[a] = base[a] ? base[a] + bb[a] + run[a] : nullptr;
-    w.vt_off = p[0]; w.vt_val = p[1]; w.vv_off = p[2]; w.vv_val = p[3];
-    w.eu_off = p[4]; w.e_w = p[5]; w.et_off = p[6]; w.et_val = p[7];
-    w.tt_off = p[8]; w.tt_val = p[9];
-    items[idx] = w;
+    write_item(m, ids, idx, mask, base, bb, run, items);
+}
+
+// Up to kBasesOne clusters: one launch, one block, which also zeroes the
+// builds' ticket counters.  (The three launches and a memset per size bin are
+// most of a small build: 16^3 grid, 128 clusters, 25.3 us a build of two
+// bins with them.)
+constexpr int kBasesOne = 1024;
+__global__ void __launch_bounds__(kBasesThreads) bases_one_kernel(DevMesh m, const int32_t *ids, int32_t n,
+                                                                  const int64_t *sizes, uint32_t mask,
+                                                                  const WorkItem *arrays_base, WorkItem *items,
+                                                                  int64_t *totals, int32_t *tickets, int nt) {
+    __shared__ int64_t s_warp[32][NA];
+    __shared__ int64_t s_tot[NA];
+    if (int(threadIdx.x) < nt) tickets[threadIdx.x] = 0;
+    int32_t *base[NA] = {arrays_base->vt_off, arrays_base->vt_val, arrays_base->vv_off, arrays_base->vv_val,
+                         arrays_base->eu_off, arrays_base->e_w,    arrays_base->et_off, arrays_base->et_val,
+                         arrays_base->tt_off, arrays_base->tt_val};
+    int64_t before[NA] = {};
+    for (int b0 = 0; b0 < n; b0 += kBasesThreads) {
+        const int idx = b0 + threadIdx.x;
+        int64_t run[NA];
+        if (idx < n) item_lengths(m, ids, sizes, mask, idx, run);
+        else
+            for (int a = 0; a < NA; ++a) run[a] = 0;
+        block_scan_na(run, s_warp, s_tot);
+        if (idx < n) write_item(m, ids, idx, mask, base, before, run, items);
+        for (int a = 0; a < NA; ++a) before[a] += s_tot[a];
+        __syncthreads();
+    }
+    if (threadIdx.x == 0)
+        for (int a = 0; a < NA; ++a) totals[a] = before[a];
 }
 
 }  // namespace
@@ -1988,21 +2027,31 @@ int launch_count_pass(const DevMesh &m, const SmemPlan &plan, const int32_t *ids
 int bases_scratch_words(int32_t n) { return ((n + kBasesThreads - 1) / kBasesThreads) * NA; }
 
 int launch_bases(const DevMesh &m, const int32_t *ids, int32_t n, const int64_t *sizes, uint32_t mask,
-                 const WorkItem *arrays_base, WorkItem *items, int64_t *totals_out, int64_t *bsum, void *stream) {
+                 const WorkItem *arrays_base, WorkItem *items, int64_t *totals_out, int64_t *bsum, int32_t *tickets,
+                 int nt, void *stream, int *launches) {
     cudaStream_t s = static_cast<cudaStream_t>(stream);
     const int nb = (n + kBasesThreads - 1) / kBasesThreads;
+    if (launches) *launches = 0;
     if (nb == 0) return 0;
-    bases_sum_kernel<<<nb, kBasesThreads, 0, s>>>(m, ids, n, sizes, mask, bsum);
+    if (nt > kBasesThreads) return int(cudaErrorInvalidValue);
+    if (n <= kBasesOne) {
+        bases_one_kernel<<<1, kBasesThreads, 0, s>>>(m, ids, n, sizes, mask, arrays_base, items, totals_out, tickets,
+                                                     nt);
+        if (launches) *launches = 1;
+        return int(cudaGetLastError());
+    }
+    bases_sum_kernel<<<nb, kBasesThreads, 0, s>>>(m, ids, n, sizes, mask, bsum, tickets, nt);
     bases_scan_kernel<<<1, kBasesThreads, 0, s>>>(nb, bsum, totals_out);
     bases_write_kernel<<<nb, kBasesThreads, 0, s>>>(m, ids, n, sizes, mask, arrays_base, bsum, items);
+    if (launches) *launches = 3;
     return int(cudaGetLastError());
 }
 
 int launch_build(const DevMesh &m, const SmemPlan &plan, const WorkItem *items, const int32_t *order, int32_t n,
                  int32_t *err, int32_t *ticket, int grid, void *stream, char *gscratch, const SmemPlan *plans,
-                 int teams) {
+                 int teams, bool reset) {
     cudaStream_t s = static_cast<cudaStream_t>(stream);
-    cudaMemsetAsync(ticket, 0, sizeof(int32_t), s);
+    if (reset) cudaMemsetAsync(ticket, 0, sizeof(int32_t), s);
     if (teams > 0) {
         if (plans || gscratch || teams > kMaxTeams || plan.threads * teams > kMaxTeamBlock)
             return int(cudaErrorInvalidValue);

@@ -11,6 +11,8 @@
 // library holds until the process exits.
 #include <cuda_runtime.h>
 
+#include <cstddef>
+
 #include <cstring>
 #include <mutex>
 #include <string>
@@ -25,12 +27,11 @@ constexpr int kMaxDevices = 64;
 
 struct NoAllocScratch {
     gale::WorkItem items[kNoAllocMaxClusters];
+    // staged by one copy, as far as the call's lists go
     gale::WorkItem base;  // the caller's ten output base pointers
-    int32_t ids[kNoAllocMaxClusters];
-    int32_t order[kNoAllocMaxClusters];
+    int32_t err, pad;     // starts at zero
+    int32_t lists[2 * kNoAllocMaxClusters];  // n ids, then the work order
     int32_t tickets[kNoAllocMaxBins];
-    int32_t err;
-    int32_t pad;
     int64_t totals[16];
     int64_t bsum[(kNoAllocMaxClusters + 255) / 256 * 10 + 16];  // output placement block sums
 };
@@ -107,49 +108,60 @@ extern "C" gale_status gale_build_clusters_noalloc(gale_ctx *ctx, const int32_t 
         }
         S = g_addr[ctx->device];
     }
-    // work order: items grouped by size bin (staged on this call's stack;
-    // the copy below has consumed it before the call returns)
-    int32_t order[kNoAllocMaxClusters];
-    int32_t cnt[kNoAllocMaxBins + 1] = {};
+    // staged on this call's stack (the copy below has consumed it before the
+    // call returns): the base pointers, a zero error word, the ids, and the
+    // work order, items grouped by size bin
+    struct Staged {
+        gale::WorkItem base;
+        int32_t err, pad;
+        int32_t lists[2 * kNoAllocMaxClusters];
+    } st;
+    static_assert(sizeof(Staged) == offsetof(NoAllocScratch, tickets) - offsetof(NoAllocScratch, base),
+                  "one copy fills the staged fields");
+    memset(&st.base, 0, sizeof(st.base));
+    st.err = st.pad = 0;
+    memcpy(st.lists, ids, sizeof(int32_t) * n);
     const int32_t nb = int32_t(ctx->bins.size());
-    for (int32_t i = 0; i < n; ++i) cnt[ctx->bin_of[ids[i]] + 1]++;
-    for (int32_t b = 0; b < nb; ++b) cnt[b + 1] += cnt[b];
-    int32_t cur[kNoAllocMaxBins];
-    for (int32_t b = 0; b < nb; ++b) cur[b] = cnt[b];
-    for (int32_t i = 0; i < n; ++i) order[cur[ctx->bin_of[ids[i]]]++] = i;
-
-    gale::WorkItem base;
-    memset(&base, 0, sizeof(base));
-    base.vt_off = (mask & GALE_VT) ? out[0] : nullptr;
-    base.vt_val = (mask & GALE_VT) ? out[1] : nullptr;
-    base.vv_off = (mask & GALE_VV) ? out[2] : nullptr;
-    base.vv_val = (mask & GALE_VV) ? out[3] : nullptr;
-    base.eu_off = (mask & GALE_ET) ? out[4] : nullptr;
-    base.e_w = (mask & GALE_ET) ? out[5] : nullptr;
-    base.et_off = (mask & GALE_ET) ? out[6] : nullptr;
-    base.et_val = (mask & GALE_ET) ? out[7] : nullptr;
-    base.tt_off = (mask & GALE_TT) ? out[8] : nullptr;
-    base.tt_val = (mask & GALE_TT) ? out[9] : nullptr;
+    gale::SmemPlan env;
+    const bool merged = gale::merged_launch(ctx, ids, n, &env);
+    int32_t *const order = st.lists + n;
+    int32_t cnt[kNoAllocMaxBins + 1] = {};
+    if (!merged) {
+        for (int32_t i = 0; i < n; ++i) cnt[ctx->bin_of[ids[i]] + 1]++;
+        for (int32_t b = 0; b < nb; ++b) cnt[b + 1] += cnt[b];
+        int32_t cur[kNoAllocMaxBins];
+        for (int32_t b = 0; b < nb; ++b) cur[b] = cnt[b];
+        for (int32_t i = 0; i < n; ++i) order[cur[ctx->bin_of[ids[i]]]++] = i;
+    }
+    {
+        const bool vt = mask & GALE_VT, vv = mask & GALE_VV, et = mask & GALE_ET, tt = mask & GALE_TT;
+        gale::WorkItem &b = st.base;
+        b.vt_off = vt ? out[0] : nullptr; b.vt_val = vt ? out[1] : nullptr;
+        b.vv_off = vv ? out[2] : nullptr; b.vv_val = vv ? out[3] : nullptr;
+        b.eu_off = et ? out[4] : nullptr; b.e_w = et ? out[5] : nullptr;
+        b.et_off = et ? out[6] : nullptr; b.et_val = et ? out[7] : nullptr;
+        b.tt_off = tt ? out[8] : nullptr; b.tt_val = tt ? out[9] : nullptr;
+    }
 
     cudaStream_t s = ctx->stream;
-    // the scratch keeps the previous call's contents: the error word must
-    // start at zero (ticket counters are reset by each launch)
-    if ((e = cudaMemsetAsync(&S->err, 0, sizeof(int32_t), s)) != cudaSuccess ||
-        (e = cudaMemcpyAsync(S->ids, ids, sizeof(int32_t) * n, cudaMemcpyHostToDevice, s)) != cudaSuccess ||
-        (e = cudaMemcpyAsync(S->order, order, sizeof(int32_t) * n, cudaMemcpyHostToDevice, s)) !=
-            cudaSuccess ||
-        (e = cudaMemcpyAsync(&S->base, &base, sizeof(base), cudaMemcpyHostToDevice, s)) != cudaSuccess)
+    const size_t staged = offsetof(Staged, lists) + sizeof(int32_t) * size_t(merged ? n : 2 * n);
+    if ((e = cudaMemcpyAsync(&S->base, &st, staged, cudaMemcpyHostToDevice, s)) != cudaSuccess)
         return fail(GALE_ECUDA, std::string("staging the work list: ") + cudaGetErrorString(e));
     const gale::DevMesh dm{ctx->d_blocks, ctx->d_blk_off, ctx->d_I_V, ctx->d_I_T, K};
     if (gale::bases_scratch_words(n) > int(sizeof(S->bsum) / sizeof(int64_t)))
         return fail(GALE_EINVAL, "placement scratch too small");
-    int rc = gale::launch_bases(dm, S->ids, n, ctx->d_sizes, mask, &S->base, S->items, S->totals, S->bsum, s);
-    for (int32_t b = 0; rc == 0 && b < nb; ++b) {
+    int rc = gale::launch_bases(dm, S->lists, n, ctx->d_sizes, mask, &S->base, S->items, S->totals, S->bsum,
+                                S->tickets, nb, s);
+    if (merged && rc == 0)
+        rc = gale::launch_build(dm, env, S->items, nullptr, n, &S->err, &S->tickets[0], n, s, nullptr, ctx->d_plans, 0,
+                                false);
+    for (int32_t b = 0; !merged && rc == 0 && b < nb; ++b) {
         const int32_t m = cnt[b + 1] - cnt[b];
         if (m == 0) continue;
         const gale::Bin &bin = ctx->bins[b];
-        rc = gale::launch_build(dm, bin.plan, S->items, S->order + cnt[b], m, &S->err, &S->tickets[b],
-                                bin.grid < m ? bin.grid : m, s, nullptr, bin.per_item ? ctx->d_plans : nullptr);
+        rc = gale::launch_build(dm, bin.plan, S->items, S->lists + n + cnt[b], m, &S->err, &S->tickets[b],
+                                bin.grid < m ? bin.grid : m, s, nullptr, bin.per_item ? ctx->d_plans : nullptr, 0,
+                                false);
     }
     if (rc != 0) return fail(GALE_ECUDA, std::string("launch: ") + cudaGetErrorString(cudaError_t(rc)));
     int32_t err = 0;
