@@ -537,6 +537,99 @@ __device__ __forceinline__ void tt_general(const Team &tm, const Smem &S, const 
 }
 
 // ---------------------------------------------------------------------------
+// A persistent CTA's next work item, taken while it builds the current one:
+// the ticket, the order entry, the item (and its plan), the block's extent
+// and the block's L2 prefetch depend on one another, a global latency each, so
+// one thread takes a step of the chain between two phases, by asynchronous
+// copies into the slot the next round reads.  (Taken in one go at the top of
+// a round, the chain stood before every block copy: phase A was 0.18 ms of a
+// 1.03 ms build of 128^3.)
+// ---------------------------------------------------------------------------
+struct NextSlot {
+    WorkItem item;
+    int64_t blk[2];  // the block's first word and its end
+    int32_t has;     // 0: no item is left
+    int32_t at;      // the claiming thread's: ticket, then position
+    int32_t step;    // ... next step (5: done)
+    int32_t pad;
+};
+
+__device__ __forceinline__ void copy_async(void *dst, const void *src, int bytes) {
+    if (bytes == 16)
+        asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(smem_addr(dst)), "l"(src) : "memory");
+    else if (bytes == 8)
+        asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"(smem_addr(dst)), "l"(src) : "memory");
+    else
+        asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(smem_addr(dst)), "l"(src) : "memory");
+}
+__device__ __forceinline__ void copies_done() { asm volatile("cp.async.wait_all;" ::: "memory"); }
+
+struct NoClaim {
+    __device__ __forceinline__ void step(int) {}
+};
+
+// (its state lives in the slot: the build has no registers to spare)
+struct NextItem {
+    const WorkItem *items;
+    const int32_t *order;
+    int32_t *ticket;
+    const SmemPlan *plans;  // NULL: the launch has one plan
+    const DevMesh &m;
+    int32_t n;
+    NextSlot *slot;
+    SmemPlan *plan;
+
+    __device__ __forceinline__ bool mine() const { return threadIdx.x == blockDim.x - 32; }
+    __device__ __forceinline__ void begin(NextSlot *s, SmemPlan *p) {
+        slot = s;
+        plan = p;
+        if (mine()) slot->step = 0;
+    }
+    __device__ __forceinline__ void step(int s) {
+        if (mine() && slot->step == s) take(s);
+    }
+    __device__ __forceinline__ void take(int s) {
+        slot->step = s + 1;
+        if (s == 0) {
+            slot->at = atomicAdd(ticket, 1);
+            return;
+        }
+        const int at = slot->at;
+        if (s == 1) {
+            slot->has = at < n;
+            slot->at = at >= n ? -1 : order ? order[at] : at;
+        } else if (at < 0) {
+            return;
+        } else if (s == 2) {
+            const char *src = reinterpret_cast<const char *>(items + at);
+            for (int i = 0; i < int(sizeof(WorkItem)); i += 16)
+                copy_async(reinterpret_cast<char *>(&slot->item) + i, src + i, 16);
+        } else if (s == 3) {
+            copies_done();
+            const int k = slot->item.k;
+            slot->blk[0] = slot->blk[1] = 0;
+            if (k < 0 || k >= m.K + m.NP) return;  // reported when its turn comes
+            copy_async(&slot->blk[0], m.blk_off + k, 8);
+            copy_async(&slot->blk[1], m.blk_off + k + 1, 8);
+            if (plans) {
+                const int32_t *src = reinterpret_cast<const int32_t *>(plans + k);
+                for (int i = 0; i < int(sizeof(SmemPlan) / 4); ++i)
+                    copy_async(reinterpret_cast<int32_t *>(plan) + i, src + i, 4);
+            }
+        } else {
+            copies_done();
+            const int64_t w0 = slot->blk[0], w1 = slot->blk[1];
+            if (w1 > w0) prefetch_l2(m.blocks + w0, uint32_t(4 * (w1 - w0)));
+        }
+    }
+    // the steps a build with fewer phases left
+    __device__ __forceinline__ void finish() {
+        if (!mine()) return;
+        for (int s = slot->step; s < 5; ++s) take(s);
+    }
+};
+
+// ---------------------------------------------------------------------------
 // One cluster.  COUNT: no output writes; sizes -> sizes_out[5].  SPILL: the
 // regions are global scratch and the rows arrive by vector loads instead of
 // the bulk copy.  `it` points to a shared-memory copy of the work item; bar
@@ -545,53 +638,57 @@ __device__ __forceinline__ void tt_general(const Team &tm, const Smem &S, const 
 // ---------------------------------------------------------------------------
 // PART: the item is a part of a cut cluster (block header part != 0); the
 // whole-cluster instances carry none of the part logic.
-template <bool COUNT, bool SPILL, bool PART, bool GEN, class Team>
+// claim: takes the CTA's next work item in steps between the phases (NextItem).
+template <bool COUNT, bool SPILL, bool PART, bool GEN, class Team, class Claim>
 __device__ bool run_cluster(const Team &tm, const DevMesh &m, const SmemPlan &plan, const Smem &S, int64_t blk_word, int64_t words,
                             uint32_t mask, const WorkItem *it, int64_t *sizes_out, int32_t *err, uint64_t *bar,
-                            uint32_t &phase) {
+                            uint32_t &phase, Claim &claim) {
     const int NT = tm.nt(), NWARP = NT >> 5;
     const int tid = tm.tid(), lane = tid & 31, warp = tid >> 5;
     const uint32_t lt = (1u << lane) - 1u;
     const Caps &caps = plan.caps;
     const int32_t *__restrict__ g = m.blocks + blk_word;
-    int32_t *flag = S.scan + flag_word(NWARP);  // [0] block fits, [1] bulk copy issued, [2] non-manifold, [3] long rows
+    int32_t *flag = S.scan + flag_word(NWARP);  // [2] non-manifold, [3] long rows
     const bool jp16 = (plan.mode & kJpos16) != 0;
 
     // ---------------- A. the block, by one bulk copy ----------------
+    // The regions that B starts from are cleared while it is under way, as
+    // far as the plan's capacities go.
+    const bool fits = words >= kHdrWords && words <= caps.blk_words && (words & 3) == 0;
+    const bool need_nb = COUNT || (mask & ~R_VT) != 0;
     if (tid == 0) {
-        const bool fits = words >= kHdrWords && words <= caps.blk_words && (words & 3) == 0;
-        int issued = 0;
-        if (fits && !SPILL) {
-            bulk_load(S.blk, g, uint32_t(4 * words), bar);
-            issued = 1;
-        }
-        flag[0] = fits;
-        flag[1] = issued;
+        if (fits && !SPILL) bulk_load(S.blk, g, uint32_t(4 * words), bar);
         flag[2] = 0;
         flag[3] = 0;
     }
-    tm.sync();
-    const bool fits = flag[0] != 0, issued = flag[1] != 0;
-    if (!fits) {
-        if (tid == 0) atomicOr(err, ERR_CAPACITY);
-        tm.sync();
-        return true;
+    claim.step(0);
+    for (int i = tid; i <= caps.nv_own; i += NT) {
+        S.c_vv[i] = 0;
+        S.vt_off[i] = 0;
     }
-    if (SPILL) {
+    if (need_nb) fill_words(tm, S.bm, caps.nv_own * plan.W, 0u);
+    fill_words(tm, reinterpret_cast<uint32_t *>(S.fill),
+               plan.stride ? (caps.nv_own * plan.stride) >> 1 : (caps.n_vt + caps.nv_own + 3) >> 1, FULL);
+    if (SPILL && fits) {
         const int4 *src = reinterpret_cast<const int4 *>(g);
         int4 *dst = reinterpret_cast<int4 *>(S.blk);
         const int n4 = int(words >> 2);
         for (int i = tid; i < n4; i += NT) dst[i] = __ldg(src + i);
-        tm.sync();
-    } else if (issued) {
-        bool ok = mbar_wait(bar, phase);
+    }
+    {
+        const bool ok = SPILL || !fits || mbar_wait(bar, phase);
         if (tm.sync_or(!ok)) {
             if (tid == 0) atomicOr(err, ERR_TIMEOUT);
             if (!ok) mbar_wait(bar, phase);  // the copy may still be in flight
             return false;
         }
-        phase ^= 1u;
     }
+    if (!fits) {
+        if (tid == 0) atomicOr(err, ERR_CAPACITY);
+        tm.sync();
+        return true;
+    }
+    if (!SPILL) phase ^= 1u;
     const BlockHdr h = *reinterpret_cast<const BlockHdr *>(S.blk);
     // a part block: its record, and the extra tmap words of its internal tets
     const PartInfo *part = (PART && h.part > 0 && h.part <= m.NP) ? m.parts + (h.part - 1) : nullptr;
@@ -648,7 +745,6 @@ __device__ bool run_cluster(const Team &tm, const DevMesh &m, const SmemPlan &pl
         b_et = __ldg(&part->b_et);
     }
 
-    const bool need_nb = COUNT || do_vv || do_et || want_tt;
     const int W = (h.nv_nb + 31) >> 5;  // bitmap words per vertex
     const int WP = W | 1;                // row stride (odd: rows start in different banks)
     uint32_t *bm = S.bm;
@@ -670,13 +766,6 @@ __device__ bool run_cluster(const Team &tm, const DevMesh &m, const SmemPlan &pl
     int32_t *const cur = reinterpret_cast<int32_t *>(S.st_v);  // fill cursors of compact rows
     auto row_at = [&](int x) -> int { return stride ? x * stride : (S.vt_off[x] + x + 1) & ~1; };
     int32_t flags = 0;
-    for (int i = tid; i <= nvo; i += NT) {
-        cnt[i] = 0;
-        S.vt_off[i] = 0;
-    }
-    if (need_nb) fill_words(tm, bm, nvo * WP, 0u);
-    fill_words(tm, reinterpret_cast<uint32_t *>(fill), stride ? (nvo * stride) >> 1 : (caps.n_vt + nvo + 3) >> 1, FULL);
-    tm.sync();
     for (int i = tid; i < n_vtets; i += NT) {
         const uint2 r = rows[i];
         const uint32_t v[4] = {r.x & 0xffffu, r.x >> 16, r.y & 0xffffu, r.y >> 16};
@@ -705,6 +794,7 @@ __device__ bool run_cluster(const Team &tm, const DevMesh &m, const SmemPlan &pl
             }
         }
     }
+    claim.step(1);
     tm.sync();
 
     // ---------------- C2. row lengths and offsets, per own vertex ----------
@@ -914,6 +1004,7 @@ __device__ bool run_cluster(const Team &tm, const DevMesh &m, const SmemPlan &pl
             tm.sync();
         }
     }
+    claim.step(2);
     if (COUNT) {
         if (tid == 0) {
             sizes_out[SZ_VT] = vt_total;
@@ -1016,6 +1107,7 @@ __device__ bool run_cluster(const Team &tm, const DevMesh &m, const SmemPlan &pl
     }
     tm.sync();
 
+    claim.step(3);
     // ---------------- C5. TT links of faces with an own lowest vertex ------
     // mask(x, w1) & mask(x, w2), less the tet's own bit, is its partner
     // across the face (x, w1, w2)
@@ -1131,6 +1223,7 @@ __device__ bool run_cluster(const Team &tm, const DevMesh &m, const SmemPlan &pl
         tm.sync();  // ET staging is dead: r1 takes the face hash
     }
 
+    claim.step(4);
     if (want_tt) {
         // ---------------- D. faces with no own vertex, against the halo ----
         const uint32_t hmask = uint32_t(caps.hcap - 1);
@@ -1285,15 +1378,17 @@ __device__ bool run_cluster(const Team &tm, const DevMesh &m, const SmemPlan &pl
 // the whole-cluster instance carries the general TT pass (E'); the hot
 // shared-memory kernel leaves it out, and the clusters that need it (the
 // counting pass marks them) run from per-item bins.
-template <bool COUNT, bool SPILL, bool GEN>
+template <bool COUNT, bool SPILL, bool GEN, class Claim>
 __device__ __forceinline__ bool run_item(bool part, const DevMesh &m, const SmemPlan &plan, const Smem &S,
                                          int64_t blk_word, int64_t words, uint32_t mask, const WorkItem *it,
-                                         int64_t *sizes_out, int32_t *err, uint64_t *bar, uint32_t &phase) {
+                                         int64_t *sizes_out, int32_t *err, uint64_t *bar, uint32_t &phase,
+                                         Claim &claim) {
     const BlockTeam tm;
     if (part)
         return run_cluster<COUNT, SPILL, true, false>(tm, m, plan, S, blk_word, words, mask, it, sizes_out, err, bar,
-                                                      phase);
-    return run_cluster<COUNT, SPILL, false, GEN>(tm, m, plan, S, blk_word, words, mask, it, sizes_out, err, bar, phase);
+                                                      phase, claim);
+    return run_cluster<COUNT, SPILL, false, GEN>(tm, m, plan, S, blk_word, words, mask, it, sizes_out, err, bar, phase,
+                                                 claim);
 }
 
 // SPILL: the cluster's regions live in a per-CTA slice of global scratch
@@ -1324,6 +1419,7 @@ __global__ void __launch_bounds__(kMaxThreads) count_kernel(DevMesh m, SmemPlan 
     __shared__ __align__(8) uint64_t s_bar;
     init_barrier<SPILL>(&s_bar);
     uint32_t phase = 0;
+    NoClaim none;
     for (;;) {
         if (threadIdx.x == 0) s_idx = atomicAdd(ticket, 1);
         __syncthreads();
@@ -1338,7 +1434,7 @@ __global__ void __launch_bounds__(kMaxThreads) count_kernel(DevMesh m, SmemPlan 
         if (threadIdx.x <= SZ_N) s_sizes[threadIdx.x] = 0;
         __syncthreads();
         if (!run_item<true, SPILL, true>(k >= m.K, m, plan, S, m.blk_off[k], m.blk_off[k + 1] - m.blk_off[k], mask, nullptr, s_sizes,
-                                      err, &s_bar, phase))
+                                      err, &s_bar, phase, none))
             return;
         __syncthreads();
         if (threadIdx.x < SZ_N) sizes[int64_t(k) * SZ_N + threadIdx.x] = s_sizes[threadIdx.x];
@@ -1351,38 +1447,27 @@ __global__ void __launch_bounds__(kMaxThreads) build_kernel(DevMesh m, SmemPlan 
                              int32_t *err, int32_t *ticket, char *gscratch) {
     extern __shared__ __align__(16) char smem[];
     const Smem S = carve(region_base<SPILL>(smem, gscratch, plan), plan);
-    __shared__ int32_t s_idx;
-    __shared__ WorkItem s_item;
+    __shared__ __align__(16) NextSlot s_slot[2];
     __shared__ __align__(8) uint64_t s_bar;
+    NextItem claim{items, order, ticket, nullptr, m, n, nullptr, nullptr};
+    claim.begin(&s_slot[0], nullptr);
+    claim.finish();
     init_barrier<SPILL>(&s_bar);
     uint32_t phase = 0;
-    if (threadIdx.x == 0) s_idx = atomicAdd(ticket, 1);
-    for (;;) {
-        __syncthreads();
-        const int idx = s_idx;
-        __syncthreads();
-        if (idx >= n) break;
-        if (threadIdx.x == 0) {
-            s_item = items[order ? order[idx] : idx];
-            s_idx = atomicAdd(ticket, 1);  // the next cluster of this CTA
-        }
-        __syncthreads();
-        if (threadIdx.x == 32 && s_idx < n) {
-            // its block into L2 while this cluster builds
-            const int k2 = items[order ? order[s_idx] : s_idx].k;
-            if (k2 >= 0 && k2 < m.K + m.NP) {
-                const int64_t w0 = m.blk_off[k2], w1 = m.blk_off[k2 + 1];
-                if (w1 > w0) prefetch_l2(m.blocks + w0, uint32_t(4 * (w1 - w0)));
-            }
-        }
-        const int k = s_item.k;
+    for (int cur = 0; s_slot[cur].has; cur ^= 1) {
+        const NextSlot &slot = s_slot[cur];
+        const int k = slot.item.k;
+        claim.begin(&s_slot[cur ^ 1], nullptr);
+        bool ok = true;
         if (k < 0 || k >= m.K + m.NP) {
             if (threadIdx.x == 0) atomicOr(err, ERR_BAD_ITEM);
-            continue;
+        } else {
+            ok = run_item<false, SPILL, SPILL>(k >= m.K, m, plan, S, slot.item.blk, slot.blk[1] - slot.blk[0],
+                                               slot.item.mask, &slot.item, nullptr, err, &s_bar, phase, claim);
         }
-        if (!run_item<false, SPILL, SPILL>(k >= m.K, m, plan, S, s_item.blk, m.blk_off[k + 1] - m.blk_off[k], s_item.mask, &s_item,
-                                       nullptr, err, &s_bar, phase))
-            return;
+        claim.finish();
+        if (!ok) return;
+        __syncthreads();
     }
 }
 
@@ -1395,6 +1480,7 @@ __global__ void __launch_bounds__(kMaxThreads) build_one_kernel(DevMesh m, SmemP
     __shared__ __align__(8) uint64_t s_bar;
     init_barrier<SPILL>(&s_bar);
     uint32_t phase = 0;
+    NoClaim none;
     if (threadIdx.x == 0) s_item = items[index];
     __syncthreads();
     if (s_item.k < 0 || s_item.k >= m.K + m.NP) {
@@ -1402,7 +1488,7 @@ __global__ void __launch_bounds__(kMaxThreads) build_one_kernel(DevMesh m, SmemP
         return;
     }
     run_cluster<false, SPILL, false, true>(BlockTeam{}, m, plan, S, s_item.blk, m.blk_off[s_item.k + 1] - m.blk_off[s_item.k], s_item.mask,
-                              &s_item, nullptr, err, &s_bar, phase);
+                              &s_item, nullptr, err, &s_bar, phase, none);
 }
 
 // ---------------------------------------------------------------------------
@@ -1429,6 +1515,7 @@ __global__ void __launch_bounds__(kMaxTeamBlock) build_kernel_team(DevMesh m, Sm
     if (tm.tid() == 0) mbar_init(&s_bar[g]);
     tm.sync();
     uint32_t phase = 0;
+    NoClaim none;
     for (;;) {
         if (tm.tid() == 0) {
             const int idx = atomicAdd(ticket, 1);
@@ -1444,7 +1531,7 @@ __global__ void __launch_bounds__(kMaxTeamBlock) build_kernel_team(DevMesh m, Sm
             continue;
         }
         if (!run_cluster<false, false, false, false>(tm, m, plan, S, s_item[g].blk, m.blk_off[k + 1] - m.blk_off[k],
-                                              s_item[g].mask, &s_item[g], nullptr, err, &s_bar[g], phase))
+                                              s_item[g].mask, &s_item[g], nullptr, err, &s_bar[g], phase, none))
             return;
         tm.sync();  // the next claim rewrites this team's item
     }
@@ -1474,6 +1561,7 @@ __global__ void __launch_bounds__(kMaxThreads) count_kernel_pi(DevMesh m, const 
     __shared__ __align__(16) SmemPlan s_plan;
     init_barrier<false>(&s_bar);
     uint32_t phase = 0;
+    NoClaim none;
     for (;;) {
         if (threadIdx.x == 0) s_idx = atomicAdd(ticket, 1);
         __syncthreads();
@@ -1490,7 +1578,7 @@ __global__ void __launch_bounds__(kMaxThreads) count_kernel_pi(DevMesh m, const 
         __syncthreads();
         const Smem S = carve(smem, s_plan);
         if (!run_item<true, false, true>(k >= m.K, m, s_plan, S, m.blk_off[k], m.blk_off[k + 1] - m.blk_off[k], mask, nullptr,
-                                      s_sizes, err, &s_bar, phase))
+                                      s_sizes, err, &s_bar, phase, none))
             return;
         __syncthreads();
         if (threadIdx.x < SZ_N) sizes[int64_t(k) * SZ_N + threadIdx.x] = s_sizes[threadIdx.x];
@@ -1502,41 +1590,29 @@ __global__ void __launch_bounds__(kMaxThreads) build_kernel_pi(DevMesh m, const 
                                                               const int32_t *order, int32_t n, int32_t *err,
                                                               int32_t *ticket) {
     extern __shared__ __align__(16) char smem[];
-    __shared__ int32_t s_idx;
-    __shared__ WorkItem s_item;
+    __shared__ __align__(16) NextSlot s_slot[2];
+    __shared__ __align__(16) SmemPlan s_plan[2];
     __shared__ __align__(8) uint64_t s_bar;
-    __shared__ __align__(16) SmemPlan s_plan;
+    NextItem claim{items, order, ticket, plans, m, n, nullptr, nullptr};
+    claim.begin(&s_slot[0], &s_plan[0]);
+    claim.finish();
     init_barrier<false>(&s_bar);
     uint32_t phase = 0;
-    if (threadIdx.x == 0) s_idx = atomicAdd(ticket, 1);
-    for (;;) {
-        __syncthreads();
-        const int idx = s_idx;
-        __syncthreads();
-        if (idx >= n) break;
-        if (threadIdx.x == 0) {
-            s_item = items[order ? order[idx] : idx];
-            s_idx = atomicAdd(ticket, 1);  // the next cluster of this CTA
-        }
-        __syncthreads();
-        if (threadIdx.x == 32 && s_idx < n) {
-            const int k2 = items[order ? order[s_idx] : s_idx].k;
-            if (k2 >= 0 && k2 < m.K + m.NP) {
-                const int64_t w0 = m.blk_off[k2], w1 = m.blk_off[k2 + 1];
-                if (w1 > w0) prefetch_l2(m.blocks + w0, uint32_t(4 * (w1 - w0)));
-            }
-        }
-        const int k = s_item.k;
+    for (int cur = 0; s_slot[cur].has; cur ^= 1) {
+        const NextSlot &slot = s_slot[cur];
+        const int k = slot.item.k;
+        claim.begin(&s_slot[cur ^ 1], &s_plan[cur ^ 1]);
+        bool ok = true;
         if (k < 0 || k >= m.K + m.NP) {
             if (threadIdx.x == 0) atomicOr(err, ERR_BAD_ITEM);
-            continue;
+        } else {
+            const Smem S = carve(smem, s_plan[cur]);
+            ok = run_item<false, false, true>(k >= m.K, m, s_plan[cur], S, slot.item.blk, slot.blk[1] - slot.blk[0],
+                                              slot.item.mask, &slot.item, nullptr, err, &s_bar, phase, claim);
         }
-        load_plan(s_plan, plans + k);
+        claim.finish();
+        if (!ok) return;
         __syncthreads();
-        const Smem S = carve(smem, s_plan);
-        if (!run_item<false, false, true>(k >= m.K, m, s_plan, S, s_item.blk, m.blk_off[k + 1] - m.blk_off[k], s_item.mask, &s_item,
-                                       nullptr, err, &s_bar, phase))
-            return;
     }
 }
 
@@ -1578,6 +1654,7 @@ __global__ void __launch_bounds__(1024) serve_kernel(DevMesh m, const SmemPlan *
     __shared__ __align__(8) uint64_t s_bar;
     init_barrier<false>(&s_bar);
     uint32_t phase = 0;
+    NoClaim none;
     unsigned long long last = globaltimer();
     __shared__ unsigned long long s_claim;
     for (;;) {
@@ -1617,7 +1694,7 @@ __global__ void __launch_bounds__(1024) serve_kernel(DevMesh m, const SmemPlan *
             __syncthreads();
             const Smem S = carve(smem, s_plan);
             go_on = run_cluster<false, false, false, true>(BlockTeam{}, m, s_plan, S, s_item.blk, m.blk_off[s_item.k + 1] - m.blk_off[s_item.k],
-                                              s_item.mask, &s_item, nullptr, err, &s_bar, phase);
+                                              s_item.mask, &s_item, nullptr, err, &s_bar, phase, none);
         } else if (threadIdx.x == 0) {
             atomicOr(err, ERR_BAD_ITEM);
         }
