@@ -775,24 +775,36 @@ __device__ bool run_cluster(const Team &tm, const DevMesh &m, const SmemPlan &pl
             q[s] = v[s] >> 5;
             bit[s] = 1u << (v[s] & 31u);
         }
+        // the four counts first: the slots they return come back while the
+        // bitmaps are set
+        int slot[4];
 #pragma unroll
         for (int s = 0; s < 4; ++s) {
             const uint32_t d = v[s] - uint32_t(lo);
+            slot[s] = stride;
             if (d < nvo_u) {
                 if (wide) {  // the halves could overflow: two counters
                     atomicAdd(&cnt[d], 3 - s);
                     atomicAdd(&S.vt_off[d + 1], 1);
                 } else {
-                    const int slot = atomicAdd(&cnt[d], 1 | ((3 - s) << 16)) & 0xffff;
-                    if (stride && slot < stride) fill[d * stride + slot] = uint16_t(keyed ? 4 * i + s : i);
+                    slot[s] = atomicAdd(&cnt[d], 1 | ((3 - s) << 16)) & 0xffff;
                 }
-                if (need_nb) {
+            }
+        }
+        if (need_nb) {
+#pragma unroll
+            for (int s = 0; s < 4; ++s) {
+                const uint32_t d = v[s] - uint32_t(lo);
+                if (d < nvo_u) {
                     uint32_t *row = bm + d * WP;
 #pragma unroll
                     for (int u = 1; u < 4; ++u) atomicOr(row + q[(s + u) & 3], bit[(s + u) & 3]);
                 }
             }
         }
+#pragma unroll
+        for (int s = 0; s < 4; ++s)
+            if (slot[s] < stride) fill[(v[s] - uint32_t(lo)) * stride + slot[s]] = uint16_t(keyed ? 4 * i + s : i);
     }
     claim.step(1);
     tm.sync();
@@ -1028,7 +1040,15 @@ __device__ bool run_cluster(const Team &tm, const DevMesh &m, const SmemPlan &pl
                 const int e0 = S.c_e[x], ne = S.c_e[x + 1] - e0;
                 const uint16_t *src = S.st_v + (S.c_vv[x + 1] & kOffMask) - ne;
                 int32_t *dst = it->e_w + e0;
-                for (int i = 0; i < ne; ++i) dst[i] = vmap[src[i]];
+                for (int i = 0; i < ne; i += 4) {  // four loads in flight
+                    const int l = ne - 1 - i;
+                    const int32_t a = vmap[src[i]], b = vmap[src[i + min(l, 1)]];
+                    const int32_t c = vmap[src[i + min(l, 2)]], d = vmap[src[i + min(l, 3)]];
+                    dst[i] = a;
+                    if (l >= 1) dst[i + 1] = b;
+                    if (l >= 2) dst[i + 2] = c;
+                    if (l >= 3) dst[i + 3] = d;
+                }
             }
             if (tid == 0) it->et_off[tot_e] = et_total + b_et;
         }
@@ -1040,14 +1060,15 @@ __device__ bool run_cluster(const Team &tm, const DevMesh &m, const SmemPlan &pl
     const int nch = plan.nch;
     uint32_t *em = S.emask;
     tm.sync();  // the VV staging and the vertex map are dead
-    // the first ET entries move from r2 to the vertex map (nvo <= nv_loc
-    // words), and the edge bases take the place of the VV offsets
-    int32_t *const et_first = S.blk + kHdrWords;
-    for (int x = tid; x < nvo; x += NT) {
-        et_first[x] = et_b[x];
-        cnt[x] = S.c_e[x] - int(uint32_t(cnt[x]) >> 24);
+    // the edge bases take the place of the VV offsets, the edge masks that of
+    // the VV staging; masks of several words also reach the first ET entries,
+    // which move to the vertex map (nvo <= nv_loc words)
+    int32_t *const et_first = nch > 1 ? S.blk + kHdrWords : et_b;
+    if (nch > 1) {
+        for (int x = tid; x < nvo; x += NT) et_first[x] = et_b[x];
+        tm.sync();
     }
-    tm.sync();  // r2 takes the edge masks
+    for (int x = tid; x < nvo; x += NT) cnt[x] = S.c_e[x] - int(uint32_t(cnt[x]) >> 24);
     fill_words(tm, em, tot_e * nch, 0u);
     tm.sync();
 
@@ -1082,23 +1103,28 @@ __device__ bool run_cluster(const Team &tm, const DevMesh &m, const SmemPlan &pl
                     j2 = (jw >> 16) & 0xffu;
                 }
                 const uint32_t x0 = v0 - uint32_t(lo), x1 = v1 - uint32_t(lo), x2 = v2 - uint32_t(lo);
+                // a tet's ranks all before its marks, so that their loads overlap
+                int e0 = 0, e1 = 0, e2 = 0;
                 uint32_t ra = 0u, rb = 0u;
                 if (x0 < nvo_u) {
-                    const int base = cnt[x0];
-                    const uint32_t a = rank(x0, v1), b = rank(x0, v2), c = rank(x0, v3);
-                    mark(base + int(a), j0);
-                    mark(base + int(b), j0);
-                    mark(base + int(c), j0);
-                    ra = a | (b << 8) | (c << 16);
+                    e0 = cnt[x0];
+                    ra = rank(x0, v1) | (rank(x0, v2) << 8) | (rank(x0, v3) << 16);
                 }
                 if (x1 < nvo_u) {
-                    const int base = cnt[x1];
-                    const uint32_t a = rank(x1, v2), b = rank(x1, v3);
-                    mark(base + int(a), j1);
-                    mark(base + int(b), j1);
-                    rb = a | (b << 8);
+                    e1 = cnt[x1];
+                    rb = rank(x1, v2) | (rank(x1, v3) << 8);
                 }
-                if (x2 < nvo_u) mark(cnt[x2] + int(rank(x2, v3)), j2);
+                if (x2 < nvo_u) e2 = cnt[x2] + int(rank(x2, v3));
+                if (x0 < nvo_u) {
+                    mark(e0 + int(ra & 0xffu), j0);
+                    mark(e0 + int((ra >> 8) & 0xffu), j0);
+                    mark(e0 + int(ra >> 16), j0);
+                }
+                if (x1 < nvo_u) {
+                    mark(e1 + int(rb & 0xffu), j1);
+                    mark(e1 + int(rb >> 8), j1);
+                }
+                if (x2 < nvo_u) mark(e2, j2);
                 if (want_tt && i >= n_ext) reinterpret_cast<uint2 *>(S.nbr)[i - n_ext] = make_uint2(ra, rb);
             }
         };
@@ -1192,10 +1218,33 @@ __device__ bool run_cluster(const Team &tm, const DevMesh &m, const SmemPlan &pl
             for (int x = tid; x < nvo; x += NT) {
                 int run = et_first[x];
                 const int e1 = S.c_e[x + 1];
-                for (int e = S.c_e[x]; e < e1; ++e) {
+                for (int e = S.c_e[x]; e < e1; e += 4) {  // four edges' masks in flight
+                    const int l = min(3, e1 - 1 - e);
+                    int n0 = 0, n1 = 0, n2 = 0, n3 = 0;
+                    for (int c = 0; c < nc; ++c) {
+                        n0 += __popc(em[e * nc + c]);
+                        n1 += __popc(em[(e + min(l, 1)) * nc + c]);
+                        n2 += __popc(em[(e + min(l, 2)) * nc + c]);
+                        n3 += __popc(em[(e + l) * nc + c]);
+                    }
                     eo[e] = run;
                     ex[e] = uint16_t(x);
-                    for (int c = 0; c < nc; ++c) run += __popc(em[e * nc + c]);
+                    run += n0;
+                    if (l >= 1) {
+                        eo[e + 1] = run;
+                        ex[e + 1] = uint16_t(x);
+                        run += n1;
+                    }
+                    if (l >= 2) {
+                        eo[e + 2] = run;
+                        ex[e + 2] = uint16_t(x);
+                        run += n2;
+                    }
+                    if (l >= 3) {
+                        eo[e + 3] = run;
+                        ex[e + 3] = uint16_t(x);
+                        run += n3;
+                    }
                 }
                 bad |= run != (x + 1 < nvo ? et_first[x + 1] : et_total);  // one distinct bit per entry
             }
@@ -1207,7 +1256,16 @@ __device__ bool run_cluster(const Team &tm, const DevMesh &m, const SmemPlan &pl
                 uint16_t *dst = S.st_et + o;
                 const uint16_t *vt = S.vt_list + S.vt_off[ex[e]] - 1;
                 for (int c = 0; c < nc; ++c) {
-                    for (uint32_t mm = em[e * nc + c]; mm; mm &= mm - 1u) *dst++ = vt[__ffs(int(mm))];
+                    for (uint32_t mm = em[e * nc + c]; mm;) {  // two entries a step
+                        const int b0 = __ffs(int(mm));
+                        mm &= mm - 1u;
+                        const int b1 = mm ? __ffs(int(mm)) : b0;
+                        const uint16_t t0 = vt[b0], t1 = vt[b1];
+                        dst[0] = t0;
+                        if (mm) dst[1] = t1;
+                        dst += mm ? 2 : 1;
+                        mm &= mm - 1u;
+                    }
                     vt += 32;
                 }
             }
@@ -1264,22 +1322,28 @@ __device__ bool run_cluster(const Team &tm, const DevMesh &m, const SmemPlan &pl
         for (int j = tid; j < h.n_halo; j += NT) {
             const int tl = n_vtets + j;
             const uint2 r = rows[tl];
+            // the faces opposite slots 0 to 3, their first probes together
+            const uint2 key[4] = {make_uint2(r.x >> 16, r.y), make_uint2(r.x & 0xffffu, r.y),
+                                  make_uint2(r.x & 0xffffu, (r.x >> 16) | (r.y & 0xffff0000u)),
+                                  make_uint2(r.x & 0xffffu, (r.x >> 16) | (r.y << 16))};
+            uint32_t hp[4], first[4];
 #pragma unroll
-            for (int f = 0; f < 4; ++f) {  // the face opposite slot f
-                const uint2 key = f == 0   ? make_uint2(r.x >> 16, r.y)
-                                  : f == 1 ? make_uint2(r.x & 0xffffu, r.y)
-                                  : f == 2 ? make_uint2(r.x & 0xffffu, (r.x >> 16) | (r.y & 0xffff0000u))
-                                           : make_uint2(r.x & 0xffffu, (r.x >> 16) | (r.y << 16));
-                uint32_t hp = face_hash(key) & hmask;
-                for (int probe = 0; probe < caps.hcap; ++probe) {
-                    const uint32_t e = hash[hp];
-                    if (e == 0u) break;
-                    if (same(e, key)) {
-                        if (atomicAdd(&hash[hp], kMatch) >= kMatch) flags |= ERR_NONMANIFOLD;
+            for (int f = 0; f < 4; ++f) {
+                hp[f] = face_hash(key[f]) & hmask;
+                first[f] = hash[hp[f]];
+            }
+#pragma unroll
+            for (int f = 0; f < 4; ++f) {
+                uint32_t e = first[f], h1 = hp[f];
+                for (int probe = 1; e != 0u; ++probe) {
+                    if (same(e, key[f])) {
+                        if (atomicAdd(&hash[h1], kMatch) >= kMatch) flags |= ERR_NONMANIFOLD;
                         S.nbr[4 * (int(e & kRefMask) - 1)] = uint16_t(tl);
                         break;
                     }
-                    hp = (hp + 1u) & hmask;
+                    if (probe == caps.hcap) break;
+                    h1 = (h1 + 1u) & hmask;
+                    e = hash[h1];
                 }
             }
         }
@@ -1296,19 +1360,28 @@ __device__ bool run_cluster(const Team &tm, const DevMesh &m, const SmemPlan &pl
         }
         // ---------------- E. TT rows ----------------
         int32_t *tcnt = S.tcnt;
-        for (int i = tid; i < n_own; i += NT) {
+        auto n_links = [&](int i) -> int {
             const uint2 nb = *reinterpret_cast<const uint2 *>(&S.nbr[i * 4]);
-            tcnt[i] = ((nb.x & 0xffffu) != 0xffffu) + ((nb.x >> 16) != 0xffffu) + ((nb.y & 0xffffu) != 0xffffu) +
-                      ((nb.y >> 16) != 0xffffu);
-        }
-        tm.sync();
-        if (COUNT && part) {
+            return ((nb.x & 0xffffu) != 0xffffu) + ((nb.x >> 16) != 0xffffu) + ((nb.y & 0xffffu) != 0xffffu) +
+                   ((nb.y >> 16) != 0xffffu);
+        };
+        const int per_t = range_len(tm, n_own);
+        const int tb0 = min(n_own, tid * per_t), tb1 = min(n_own, tb0 + per_t);
+        int mine_tt = 0;
+        for (int i = tb0; i < tb1; ++i) {
+            const int c = n_links(i);
+            mine_tt += c;
             // row lengths of the part's own internal tets, by canonical id
-            for (int i = tid; i < n_own; i += NT)
-                if ((rows[n_ext + i].x & 0xffffu) - uint32_t(lo) < nvo_u) m.tt_pos[gtet(n_ext + i)] = tcnt[i];
-            tm.sync();
+            if (COUNT && part && (rows[n_ext + i].x & 0xffffu) - uint32_t(lo) < nvo_u) m.tt_pos[gtet(n_ext + i)] = c;
         }
-        const int tot_tt = block_scan_array(tm, tcnt, n_own, S.scan);
+        int tot_tt;
+        int run_tt = block_scan_thread(tm, mine_tt, S.scan, &tot_tt);
+        if (!COUNT && !part)
+            for (int i = tb0; i < tb1; ++i) {
+                tcnt[i] = run_tt;
+                run_tt += n_links(i);
+            }
+        tm.sync();
         if (COUNT) {
             if (tid == 0) sizes_out[SZ_TT] = tot_tt;
         } else if (part) {
@@ -1981,11 +2054,13 @@ SmemPlan plan_smem(const Caps &c, int threads) {
         // word each) end with nbr and reach back into what r2 leaves free.
         const int64_t vv = a16(std::max(2 * int64_t(c.max_vv), 4 * nvo)), eb = a16(4 * nvo);
         const int64_t lr = c.max_deg > 32 ? a16(2 * nvo) : 0;
-        p.r2 = take(std::max<int64_t>(4 * int64_t(c.max_e) * p.nch, vv + eb + lr));
-        p.et_b = int32_t(p.r2 + vv);
-        p.long_rows = int32_t(p.r2 + vv + eb);
+        const int64_t em = 4 * int64_t(c.max_e) * p.nch;
+        const int64_t eb0 = p.nch == 1 ? std::max(vv, a16(em)) : vv;  // single-word masks leave the ET entries in place
+        p.r2 = take(std::max<int64_t>(em, eb0 + eb + lr));
+        p.et_b = int32_t(p.r2 + eb0);
+        p.long_rows = int32_t(p.r2 + eb0 + eb);
         const int64_t n_fill = a16(p.stride ? 2 * nvo * p.stride : 2 * (int64_t(c.n_vt) + nvo + 4));
-        p.nbr = take(std::max(8 * int64_t(c.n_own), p.r2 + vv + eb + lr + n_fill - off));
+        p.nbr = take(std::max(8 * int64_t(c.n_own), p.r2 + eb0 + eb + lr + n_fill - off));
         p.fill = int32_t(std::min<int64_t>(off - n_fill, INT32_MAX));
         // r1: bitmaps + rank prefixes | ET staging + the edges' lower vertices
         // | face hash + TT counts + TT staging
