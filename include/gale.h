@@ -311,7 +311,7 @@ gale_status gale_copy_to_host(gale_ctx *ctx, void *dst, const void *src, size_t 
  *   host_dst  one buffer per array of mask, laid out as a bulk build lays
  *             out the device arrays (lengths as gale_bulk_arrays reports after
  *             the call); pinned memory is needed for the overlap.
- *   chunks    0 = automatic (about 256 MB of output per chunk, at most 16),
+ *   chunks    0 = automatic (the root of the output over 20 MB, at most 16),
  *             else 1..64.
  * Afterwards the device bulk arrays hold the same result as after
  * gale_build_clusters(ctx, ids, n, mask, GALE_MODE_BATCHED).  Blocks until

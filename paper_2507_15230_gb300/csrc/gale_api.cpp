@@ -1,6 +1,8 @@
 // C ABI: context life cycle, loading, bulk builds, views and exports.
 #include <cuda_runtime.h>
 
+#include <cmath>
+
 #include <algorithm>
 #include <atomic>
 #include <chrono>
@@ -986,33 +988,41 @@ gale_status gale_build_clusters(gale_ctx *ctx, const int32_t *ids, int32_t n, ui
     const bool all = (ids == nullptr || n <= 0);
     const int32_t cnt = all ? K : n;
     if (!all && n > K) return fail(GALE_EINVAL, "more ids than clusters");
-    std::vector<int32_t> list(cnt);
-    if (all) {
-        std::iota(list.begin(), list.end(), 0);
-    } else {
-        std::vector<uint8_t> seen(K, 0);
-        for (int32_t i = 0; i < n; ++i) {
-            if (ids[i] < 0 || ids[i] >= K) return fail(GALE_EINVAL, "cluster id out of range");
-            if (seen[ids[i]]++) return fail(GALE_EINVAL, "cluster id listed twice");
-            list[i] = ids[i];
+    std::vector<int32_t> list;
+    // a full build's placement is the context's: made once per relation mask
+    // in a row (at 256^3 0.7 ms a call on the host)
+    const bool placed = all && mode == GALE_MODE_BATCHED && ctx->bulk_full && ctx->bulk_mask == mask;
+    if (!placed) {
+        list.resize(cnt);
+        if (all) {
+            std::iota(list.begin(), list.end(), 0);
+        } else {
+            std::vector<uint8_t> seen(K, 0);
+            for (int32_t i = 0; i < n; ++i) {
+                if (ids[i] < 0 || ids[i] >= K) return fail(GALE_EINVAL, "cluster id out of range");
+                if (seen[ids[i]]++) return fail(GALE_EINVAL, "cluster id listed twice");
+                list[i] = ids[i];
+            }
         }
-    }
-    // placement bookkeeping on the host (views); the device recomputes it
-    ctx->bulk_offs.assign(size_t(cnt) * 10, 0);
-    int64_t run[10] = {};
-    for (int32_t i = 0; i < cnt; ++i) {
-        int64_t L[10];
-        gale::item_lengths(ctx, list[i], mask, L);
-        for (int a = 0; a < 10; ++a) {
-            ctx->bulk_offs[size_t(i) * 10 + a] = run[a];
-            run[a] += L[a];
+        // placement bookkeeping on the host (views); the device recomputes it
+        ctx->bulk_full = false;
+        ctx->bulk_offs.assign(size_t(cnt) * 10, 0);
+        int64_t run[10] = {};
+        for (int32_t i = 0; i < cnt; ++i) {
+            int64_t L[10];
+            gale::item_lengths(ctx, list[i], mask, L);
+            for (int a = 0; a < 10; ++a) {
+                ctx->bulk_offs[size_t(i) * 10 + a] = run[a];
+                run[a] += L[a];
+            }
         }
+        gale_status st = ensure_bulk(ctx, run);
+        if (st != GALE_OK) return st;
+        for (int a = 0; a < 10; ++a) ctx->bulk_len[a] = run[a];
+        ctx->bulk_ids = list;
+        ctx->bulk_mask = mask;
+        ctx->bulk_full = all;
     }
-    gale_status st = ensure_bulk(ctx, run);
-    if (st != GALE_OK) return st;
-    for (int a = 0; a < 10; ++a) ctx->bulk_len[a] = run[a];
-    ctx->bulk_ids = list;
-    ctx->bulk_mask = mask;
     const gale::DevMesh dm = dev_mesh(ctx);
     const WorkItem *base = ctx->d_arrays_base + mask;
     int64_t launches = 0;
@@ -1198,6 +1208,7 @@ gale_status gale_build_export(gale_ctx *ctx, const int32_t *ids, int32_t n, uint
     const uint32_t rel_of[10] = {GALE_VT, GALE_VT, GALE_VV, GALE_VV, GALE_ET, GALE_ET, GALE_ET, GALE_ET, GALE_TT, GALE_TT};
     for (int a = 0; a < 10; ++a)
         if ((mask & rel_of[a]) && !h[a]) return fail(GALE_EINVAL, "NULL host buffer for a requested array");
+    ctx->bulk_full = false;
     // placement of every listed cluster, and the chunk boundaries: about
     // equal output bytes per chunk
     ctx->bulk_offs.assign(size_t(cnt) * 10, 0);
@@ -1219,9 +1230,14 @@ gale_status gale_build_export(gale_ctx *ctx, const int32_t *ids, int32_t n, uint
     for (int a = 0; a < 10; ++a) ctx->bulk_len[a] = run[a];
     ctx->bulk_ids = list;
     ctx->bulk_mask = mask;
-    // automatic: one chunk per 256 MB of output, at most 16 (measured at
-    // 256^3: 16 chunks 44.4 ms, 8 chunks 44.8 ms, 4 chunks 45.7 ms)
-    if (chunks == 0) chunks = int32_t(std::min<int64_t>(16, std::max<int64_t>(1, bytes_before[cnt] >> 28)));
+    // automatic: the build of the first chunk is exposed, a further chunk costs
+    // ten more copies, so the best count grows with the root of the output.
+    // Measured (ms by chunk count): 430 MB 1: 3.09, 2: 2.77, 4: 2.63, 6: 2.61,
+    // 12: 2.68; 1.0 GB 1: 6.39, 4: 5.84, 6: 5.79, 12: 5.85; 127 MB 1: 0.90,
+    // 2: 0.87, 6: 0.91; 31 MB 1: 0.29, 2: 0.28, 4: 0.31; 8.1 GB 4: 45.7,
+    // 8: 44.8, 16: 44.4
+    if (chunks == 0)
+        chunks = std::max(1, std::min(16, int32_t(std::lround(std::sqrt(double(bytes_before[cnt]) / 20e6)))));
     chunks = std::max(1, std::min(chunks, cnt));
     std::vector<int32_t> cut(size_t(chunks) + 1, cnt);
     cut[0] = 0;
@@ -1472,6 +1488,7 @@ gale_status gale_autotune(gale_ctx *ctx, uint32_t mask, int32_t reps, float *bes
     const int32_t K = ctx->hm.K;
     // outputs of every cluster: one placement pass, then bins are timed alone
     int64_t run[10] = {};
+    ctx->bulk_full = false;
     ctx->bulk_offs.assign(size_t(K) * 10, 0);
     for (int32_t k = 0; k < K; ++k) {
         int64_t L[10];

@@ -101,6 +101,7 @@ struct gale_ctx {
     std::vector<int64_t> bulk_offs;  // [n*10]
     std::vector<int32_t> bulk_ids;
     uint32_t bulk_mask = 0;
+    bool bulk_full = false;  // the fields above describe a full build under bulk_mask
 
     // streams and events that several size bins' launches fork to and join by
     std::vector<cudaStream_t> bin_streams;
