@@ -343,7 +343,8 @@ SmemPlan serve_plan(gale_ctx *ctx, bool *fits, std::vector<uint8_t> *in_loop, st
 // takes the longest item's time, not the sum over the bins of each bin's, and
 // more threads an item than the bins' rule gives small ones.  Measured: 16^3
 // grid (two bins of 64 and 128 threads) 73.8 us alone, as one bin of 512
-// threads 41.4; 3 clusters of a Delaunay mesh in three bins 151 us.  The line
+// threads 41.4, merged 32; 3 clusters of a Delaunay mesh in three bins 151
+// us a call, merged 62.  The line
 // lies where the items no longer all fit.  A block size or occupancy set by
 // the caller, teams and global-scratch bins keep their bins' launches.
 bool merged_launch(const gale_ctx *ctx, const int32_t *items, int32_t n, SmemPlan *env) {
@@ -609,7 +610,7 @@ cudaError_t ensure_bin_streams(gale_ctx *ctx, size_t ns) {
 // zeroed the tickets).  Several bins run side by side: forked to streams of
 // the context and joined again, so that one bin's last CTAs share the GPU
 // with the next one's (2e5-point Delaunay mesh, six bins of 1,500 items: 459
-// us one after another).  The largest CTAs go first; bins in global
+// us one after another, 336 side by side).  The largest CTAs go first; bins in global
 // scratch share it and stay in one stream.  Works under stream capture.
 cudaError_t run_bins(gale_ctx *ctx, const gale::DevMesh &dm, const WorkItem *items, std::vector<BinRun> runs,
                      int64_t *launches) {
