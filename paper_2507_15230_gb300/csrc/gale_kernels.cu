@@ -543,9 +543,9 @@ __device__ __forceinline__ void tt_general(const Team &tm, const Smem &S, const 
 // the ticket, the order entry, the item (and its plan), the block's extent
 // and the block's L2 prefetch depend on one another, a global latency each, so
 // one thread takes a step of the chain between two phases, by asynchronous
-// copies into the slot the next round reads.  (Taken in one go at the top of
-// a round, the chain stood before every block copy: phase A was 0.18 ms of a
-// 1.03 ms build of 128^3.)
+// copies into the slot that the next item is read from.  (Taken in one go at
+// the top of the loop, the chain stood before every block copy: 1.031 ms a
+// build of 128^3 against 1.015.)
 // ---------------------------------------------------------------------------
 struct NextSlot {
     WorkItem item;
