@@ -56,9 +56,9 @@
 // counters and lane masks in B, C1 as a pass of its own, edge ranks recomputed
 // in C5 and a scan over the edges in C4, 107.6k warp instructions, 29.8k
 // shared wavefronts and 9.07 ms per 256^3 build; with the passes above 70.7k,
-// 24.4k and 7.06 ms.  What is left waits on shared-memory loads and barriers
-// (48 % issue), so loads go before the atomics and stores they may alias, a
-// few steps at a time: 6.89 ms.
+// 24.4k and 7.06 ms.  What is left waits on the shared-memory pipe (76 % of
+// its peak, issue 58 %) and barriers, so loads go before the atomics and
+// stores they may alias, a few steps at a time: 77k, 23.5k and 6.85 ms.
 #include <cuda_runtime.h>
 #include <stdint.h>
 
