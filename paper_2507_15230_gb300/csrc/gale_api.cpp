@@ -245,9 +245,15 @@ gale_status plan_bins(gale_ctx *ctx, bool with_sizes) {
     if (int(ctx->bins.size()) > gale::kMaxBins)
         return fail(GALE_EINVAL, "the working sets fall into more than " + std::to_string(gale::kMaxBins) +
                                      " size bins; use more even clusters");
+    // what launches ask for: the bins' plans, and (merged launches) any
+    // member's own, which can be the larger: a bin's maxima may take its
+    // padded rows away
     int max_total = 0;
-    for (auto &b : ctx->bins)
-        if (!b.spill) max_total = std::max(max_total, b.plan.total);
+    for (auto &b : ctx->bins) {
+        if (b.spill) continue;
+        max_total = std::max(max_total, b.plan.total);
+        for (int32_t k : b.clusters) max_total = std::max(max_total, ctx->h_plans[k].total);
+    }
     if (!gale::prepare_kernels(max_total))
         return fail(GALE_ECUDA, "setting the kernels' shared memory limit failed");
     int64_t spill_need = 0;
