@@ -111,6 +111,8 @@ gale_status plan_bins(gale_ctx *ctx, bool with_sizes) {
     auto caps_k = [&](int32_t k) {
         return gale::caps_of(ctx->hm.stats[k], with_sizes ? ctx->sizes.data() + size_t(5) * k : nullptr);
     };
+    // an item's own plan (parts, held well under a CTA's limit, have no tight one)
+    auto plan_k = [&](int32_t k, int threads) { return gale::plan_smem(caps_k(k), threads, k < K); };
     std::vector<int32_t> need(NI), thr(NI);
     std::vector<uint8_t> big(NI), cut(NI, 0), gen(NI, 0);
     for (int32_t k = 0; k < NI; ++k) {
@@ -118,8 +120,9 @@ gale_status plan_bins(gale_ctx *ctx, bool with_sizes) {
             return fail(GALE_EINVAL, "cluster " + std::to_string(k < K ? k : ctx->hm.parts[k - K].k) +
                                          " has a vertex with more than 255 upper neighbours (unsupported)");
         thr[k] = threads_for(ctx, ctx->hm.stats[k]);
-        need[k] = gale::plan_smem(caps_k(k), thr[k]).total;
+        need[k] = plan_k(k, thr[k]).total;
         big[k] = std::max<int64_t>(need[k], gale::class_bytes(caps_k(k), thr[k])) > smem_cta;
+        if (big[k]) need[k] = gale::plan_smem(caps_k(k), thr[k], false).total;
         if (k < K) cut[k] = ctx->hm.part_first[k + 1] > ctx->hm.part_first[k];
         if (with_sizes && k < K && size_t(k) < ctx->tt_general.size()) gen[k] = ctx->tt_general[k] != 0 && !big[k];
     }
@@ -143,7 +146,7 @@ gale_status plan_bins(gale_ctx *ctx, bool with_sizes) {
     auto close = [&]() {
         if (members.empty()) return;
         gale::Bin b;
-        b.plan = gale::plan_smem(cur, cur_thr);
+        b.plan = gale::plan_smem(cur, cur_thr, !cur_big && members[0] < K);
         b.spill = cur_big;
         b.cut = cur_cut;
         b.tt_general = cur_gen;
@@ -167,15 +170,20 @@ gale_status plan_bins(gale_ctx *ctx, bool with_sizes) {
         cur_gen = gen[k];
         gale::Caps m = members.empty() ? caps_k(k) : merge(cur, caps_k(k));
         if (!cur_big) {
-            int tot = gale::plan_smem(m, cur_thr).total;
-            while (tier < tiers.size() && tot > tiers[tier]) {
+            gale::SmemPlan p = members.empty() ? plan_k(k, cur_thr) : gale::plan_smem(m, cur_thr);
+            if (!members.empty() && (p.mode & gale::kTight)) {  // the tight layout is an item's own
+                close();
+                m = caps_k(k);
+                p = plan_k(k, cur_thr);
+            }
+            while (tier < tiers.size() && p.total > tiers[tier]) {
                 close();
                 ++tier;
                 m = caps_k(k);
-                tot = gale::plan_smem(m, cur_thr).total;
+                p = plan_k(k, cur_thr);
             }
             if (tier >= tiers.size()) tier = tiers.size() - 1;
-        } else if (!members.empty() && gale::plan_smem(m, cur_thr).total > 2 * need[k]) {
+        } else if (!members.empty() && gale::plan_smem(m, cur_thr, false).total > 2 * need[k]) {
             // spill bins: keep the merged plan within twice a member's own
             close();
             m = caps_k(k);
@@ -192,7 +200,7 @@ gale_status plan_bins(gale_ctx *ctx, bool with_sizes) {
     // shared memory).
     ctx->h_plans.assign(size_t(NI), gale::SmemPlan{});
     if (with_sizes)
-        for (int32_t k = 0; k < NI; ++k) ctx->h_plans[k] = gale::plan_smem(caps_k(k), thr[k]);
+        for (int32_t k = 0; k < NI; ++k) ctx->h_plans[k] = plan_k(k, thr[k]);
     {
         // (block size, bin of cut clusters) -> bins of the top tier
         using Key = std::pair<int, bool>;
@@ -202,8 +210,9 @@ gale_status plan_bins(gale_ctx *ctx, bool with_sizes) {
         std::vector<gale::Bin> kept;
         std::map<Key, gale::Bin> top;  // merged bins
         for (auto &b : ctx->bins) {
-            if (b.tt_general) {  // each member under its own plan, in build_kernel_pi
-                for (int32_t k : b.clusters) ctx->h_plans[k] = gale::plan_smem(caps_k(k), b.plan.threads);
+            const bool lone_tight = !b.spill && (b.plan.mode & gale::kTight) && ntop[Key(b.plan.threads, b.cut)] < 2;
+            if (b.tt_general || lone_tight) {  // each member under its own plan, in build_kernel_pi
+                for (int32_t k : b.clusters) ctx->h_plans[k] = plan_k(k, b.plan.threads);
                 b.per_item = true;
                 kept.push_back(std::move(b));
                 continue;
@@ -216,7 +225,7 @@ gale_status plan_bins(gale_ctx *ctx, bool with_sizes) {
             t.cut = b.cut;
             const bool first = t.clusters.empty();
             for (int32_t k : b.clusters) {
-                ctx->h_plans[k] = gale::plan_smem(caps_k(k), b.plan.threads);
+                ctx->h_plans[k] = plan_k(k, b.plan.threads);
                 if (first && t.clusters.empty()) t.plan = ctx->h_plans[k];
                 else t.plan.caps = merge(t.plan.caps, ctx->h_plans[k].caps);
                 t.plan.total = std::max(t.plan.total, ctx->h_plans[k].total);
@@ -261,6 +270,7 @@ gale_status plan_bins(gale_ctx *ctx, bool with_sizes) {
         int per_sm = gale::max_ctas_per_sm(b.plan, b.spill, b.per_item);
         if (per_sm < 1 && !b.spill && !b.per_item) {
             b.spill = true;  // cannot launch with this much shared memory: run in global scratch
+            b.plan = gale::plan_smem(b.plan.caps, b.plan.threads, false);
             per_sm = gale::max_ctas_per_sm(b.plan, true);
         }
         if (per_sm < 1) return fail(GALE_EINVAL, "a size bin cannot be launched (threads or registers)");
@@ -1456,7 +1466,7 @@ gale_status gale_set_teams(gale_ctx *ctx, int32_t team_threads, int32_t teams) {
             b.teams = 0;
             continue;
         }
-        const gale::SmemPlan p = gale::plan_smem(b.plan.caps, team_threads);
+        const gale::SmemPlan p = gale::plan_smem(b.plan.caps, team_threads, false);
         if (int64_t(p.total) * teams > smem_limit) continue;
         max_total = std::max(max_total, p.total * teams);
         if (!gale::prepare_kernels(max_total)) return fail(GALE_ECUDA, "setting the kernels' shared memory limit failed");
@@ -1534,13 +1544,13 @@ gale_status gale_autotune(gale_ctx *ctx, uint32_t mask, int32_t reps, float *bes
         int best_grid = bin.grid, best_per = bin.ctas_per_sm;
         std::vector<gale::SmemPlan> best_members;
         for (int T : cand_threads) {
-            gale::SmemPlan plan = gale::plan_smem(bin.plan.caps, T);
+            gale::SmemPlan plan = gale::plan_smem(bin.plan.caps, T, (bin.plan.mode & gale::kTight) != 0);
             if (bin.per_item) {
                 // the members' own plans at this block size; the envelope
                 // takes the largest shared memory
                 int top = 0;
                 for (int32_t k : bin.clusters) {
-                    ctx->h_plans[k] = gale::plan_smem(bin_caps(ctx, k), T);
+                    ctx->h_plans[k] = gale::plan_smem(bin_caps(ctx, k), T, k < K);
                     top = std::max(top, ctx->h_plans[k].total);
                 }
                 plan.threads = T;
@@ -1614,7 +1624,7 @@ gale_status gale_autotune(gale_ctx *ctx, uint32_t mask, int32_t reps, float *bes
             for (int T : {32, 64, 128})
                 for (int tm : {2, 4, 8}) {
                     if (T * tm > 512) continue;
-                    const gale::SmemPlan plan = gale::plan_smem(bin.plan.caps, T);
+                    const gale::SmemPlan plan = gale::plan_smem(bin.plan.caps, T, false);
                     if (int64_t(plan.total) * tm > smem_limit) continue;
                     const int per = gale::max_ctas_per_sm_teams(plan, tm);
                     if (per < 1) continue;

@@ -163,7 +163,9 @@ struct Caps {
 //       the per-edge tet masks;
 //   r1: the neighbour bitmaps and their rank prefixes; then ET staging; then
 //       the boundary-face hash, the TT counts and the TT staging.
-constexpr int32_t kKeyed = 1, kJpos16 = 2;
+// Tight plans (kTight) fill and sort VT's rows in place and keep neither the
+// first ET entries nor long rows.
+constexpr int32_t kKeyed = 1, kJpos16 = 2, kTight = 4;
 struct SmemPlan {
     int32_t threads;
     int32_t W;          // row stride (words, odd) of the neighbour bitmaps
@@ -171,8 +173,9 @@ struct SmemPlan {
     int32_t stride;     // row stride of the padded rows (uint16s; 0: compact rows)
     int32_t fill;       // the rows in arrival order (inside r2 and nbr)
     int32_t mode;       // kKeyed: the rows' entries carry the vertex's slot in the tet;
-                        // kJpos16: VT rows may exceed 256 entries, positions are 16-bit
-    int32_t scan;       // scan scratch and flags
+                        // kJpos16: VT rows may exceed 256 entries, positions are 16-bit;
+                        // kTight: the smallest layout (kernels that carry the rare forms)
+    int32_t scan;       // scan scratch
     int32_t blk;        // int32[blk_words] the cluster's block (bulk copy)
     int32_t vt_off;     // int32[nv_own+1]
     int32_t vt_list;    // uint16[n_vt]
@@ -203,21 +206,29 @@ enum : int32_t {
     ERR_BAD_BLOCK = 32,    // a block broke an invariant of its layout
 };
 
-SmemPlan plan_smem(const Caps &c, int threads);
+// Layout of a build.  shared: for shared memory, where a plan that would pass
+// kCompactFit takes the tight layout if that fits (global scratch has room).
+SmemPlan plan_smem(const Caps &c, int threads, bool shared = true);
 // Capacities of one cluster or part; staging capacities come from the exact
 // sizes of the counting pass (sizes == nullptr: a counting plan, no staging).
 Caps caps_of(const ClusterStat &s, const int64_t *sizes);
 // Size class of a working set, in bytes.  It draws the lines that callers
 // see: which clusters are cut into parts, and which run from global scratch
 // (and are refused by gale_build_clusters_noalloc).  It is the shared memory
-// of a build with counters and lane masks per warp in phase B; a build plan
-// near a CTA's limit (plan_smem) needs no more than that.
+// of a build with counters and lane masks per warp in phase B.  The plans of
+// plan_smem may take more (rows in arrival order beside VT's, positions shared
+// with edge offsets), the tight layout never does, so a class that fits a CTA
+// has a plan that does.
 int64_t class_bytes(const Caps &c, int threads);
 // ... with the staged rows' sizes from estimates (before the counting pass).
 int64_t estimate_class(const ClusterStat &s, int threads);
 
-// Padded rows are given up where the plan with them would pass this.
+// Padded rows are given up where the plan with them would pass kPaddedFit,
+// compact ones where it would pass kCompactFit: a CTA's 227 KB less the
+// kernels' static shared memory (1,632 bytes at most; see dynamic_smem_limit).
 constexpr int64_t kPaddedFit = 220 * 1024;
+constexpr int64_t kCtaBytes = 227 * 1024;
+constexpr int64_t kCompactFit = kCtaBytes - 1664;
 
 // Size bins a context may have (one ticket counter each in the build and
 // serving paths).

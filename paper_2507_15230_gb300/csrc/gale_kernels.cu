@@ -72,10 +72,9 @@ namespace gale {
 
 namespace {
 
-// scan scratch: block_scan4's words, and four flags in those that blocks of
-// up to 27 warps leave free
-constexpr int scan_words(int threads) { return threads <= 864 ? 128 : 140; }
-GALE_HD constexpr int flag_word(int warps) { return warps <= 27 ? 28 : 136; }
+constexpr int kScanWords = 128;  // scan scratch: a word per warp (up to 32) and value
+// words of the block's header, free once every thread has read it
+constexpr int kFlagNonManifold = 0, kFlagLong = 1, kScanTotals = 4;
 constexpr unsigned FULL = 0xffffffffu;
 constexpr int kWaitLimit = 1 << 22;  // polls of the block copy's barrier before giving up
 
@@ -232,13 +231,12 @@ __device__ __forceinline__ int block_scan_thread(const Team &tm, int v, int32_t 
 }
 
 // Exclusive scans of four values per thread over the team, in place; totals
-// to t[0..3].  scr needs 128 words (136 with 32 warps).
+// to t[0..3], by way of tot[0..3].  scr needs kScanWords words.
 template <class Team>
-__device__ __forceinline__ void block_scan4(const Team &tm, int &a, int &b, int &c, int &d, int32_t *scr, int *t) {
+__device__ __forceinline__ void block_scan4(const Team &tm, int &a, int &b, int &c, int &d, int32_t *scr, int32_t *tot,
+                                            int *t) {
     const int nw = tm.nt() >> 5;
     const int lane = tm.tid() & 31, warp = tm.tid() >> 5;
-    int32_t *const tot = nw < 32 ? scr + nw : scr + 128;
-    const int ts = nw < 32 ? 32 : 1;
     const int ia = warp_incl_scan(a, lane), ib = warp_incl_scan(b, lane);
     const int ic = warp_incl_scan(c, lane), id = warp_incl_scan(d, lane);
     if (lane == 31) {
@@ -252,11 +250,11 @@ __device__ __forceinline__ void block_scan4(const Team &tm, int &a, int &b, int 
         const int w = lane < nw ? scr[32 * s + lane] : 0;
         const int wi = warp_incl_scan(w, lane);
         if (lane < nw) scr[32 * s + lane] = wi - w;
-        if (lane == 31) tot[ts * s] = wi;
+        if (lane == 31) tot[s] = wi;
     }
     tm.sync();
 #pragma unroll
-    for (int s = 0; s < 4; ++s) t[s] = tot[ts * s];
+    for (int s = 0; s < 4; ++s) t[s] = tot[s];
     a = scr[warp] + ia - a;
     b = scr[32 + warp] + ib - b;
     c = scr[64 + warp] + ic - c;
@@ -639,7 +637,9 @@ struct NextItem {
 // false when a bounded wait ran out (the CTA must stop).
 // ---------------------------------------------------------------------------
 // PART: the item is a part of a cut cluster (block header part != 0); the
-// whole-cluster instances carry none of the part logic.
+// whole-cluster instances carry none of the part logic.  GEN: the instance
+// carries the rare forms of whole clusters (E', tight plans), which the hot
+// shared-memory kernel leaves out.
 // claim: takes the CTA's next work item in steps between the phases (NextItem).
 template <bool COUNT, bool SPILL, bool PART, bool GEN, class Team, class Claim>
 __device__ bool run_cluster(const Team &tm, const DevMesh &m, const SmemPlan &plan, const Smem &S, int64_t blk_word, int64_t words,
@@ -647,30 +647,27 @@ __device__ bool run_cluster(const Team &tm, const DevMesh &m, const SmemPlan &pl
                             uint32_t &phase, Claim &claim) {
     const int NT = tm.nt(), NWARP = NT >> 5;
     const int tid = tm.tid(), lane = tid & 31, warp = tid >> 5;
-    const uint32_t lt = (1u << lane) - 1u;
     const Caps &caps = plan.caps;
     const int32_t *__restrict__ g = m.blocks + blk_word;
-    int32_t *flag = S.scan + flag_word(NWARP);  // [2] non-manifold, [3] long rows
+    int32_t *const flag = S.blk;  // kFlag* words
     const bool jp16 = (plan.mode & kJpos16) != 0;
+    const bool tight = GEN && !SPILL && (plan.mode & kTight) != 0;
 
     // ---------------- A. the block, by one bulk copy ----------------
     // The regions that B starts from are cleared while it is under way, as
     // far as the plan's capacities go.
     const bool fits = words >= kHdrWords && words <= caps.blk_words && (words & 3) == 0;
     const bool need_nb = COUNT || (mask & ~R_VT) != 0;
-    if (tid == 0) {
-        if (fits && !SPILL) bulk_load(S.blk, g, uint32_t(4 * words), bar);
-        flag[2] = 0;
-        flag[3] = 0;
-    }
+    if (tid == 0 && fits && !SPILL) bulk_load(S.blk, g, uint32_t(4 * words), bar);
     claim.step(0);
     for (int i = tid; i <= caps.nv_own; i += NT) {
         S.c_vv[i] = 0;
         S.vt_off[i] = 0;
     }
     if (need_nb) fill_words(tm, S.bm, caps.nv_own * plan.W, 0u);
-    fill_words(tm, reinterpret_cast<uint32_t *>(S.fill),
-               plan.stride ? (caps.nv_own * plan.stride) >> 1 : (caps.n_vt + caps.nv_own + 3) >> 1, FULL);
+    if (!tight)
+        fill_words(tm, reinterpret_cast<uint32_t *>(S.fill),
+                   plan.stride ? (caps.nv_own * plan.stride) >> 1 : (caps.n_vt + caps.nv_own + 3) >> 1, FULL);
     if (SPILL && fits) {
         const int4 *src = reinterpret_cast<const int4 *>(g);
         int4 *dst = reinterpret_cast<int4 *>(S.blk);
@@ -759,7 +756,9 @@ __device__ bool run_cluster(const Team &tm, const DevMesh &m, const SmemPlan &pl
     // are ORed into x's bitmap.  With padded rows (plan.stride) the value the
     // count returns is also the tet's slot; otherwise a second pass fills
     // compact rows by cursors.  An entry is 4 * tet + x's slot in the tet
-    // (kKeyed).
+    // (kKeyed).  Tight plans have no room for these rows beside VT's own
+    // (kTight): they fill VT in place, with its offsets as the cursors, and a
+    // warp then sorts each row there; the first ET entries are not kept.
     int32_t *const cnt = S.c_vv;  // the counters, then VV offsets, then the biased edge bases
     int32_t *const et_b = S.et_b;  // first ET entry of each own vertex
     const int stride = plan.stride;
@@ -810,6 +809,10 @@ __device__ bool run_cluster(const Team &tm, const DevMesh &m, const SmemPlan &pl
     }
     claim.step(1);
     tm.sync();
+    if (tid == 0) {  // every thread has read the header
+        flag[kFlagNonManifold] = 0;
+        flag[kFlagLong] = 0;
+    }
 
     // ---------------- C2. row lengths and offsets, per own vertex ----------
     // Every bitmap word gets the number of neighbours before it (8 bits); the
@@ -827,7 +830,7 @@ __device__ bool run_cluster(const Team &tm, const DevMesh &m, const SmemPlan &pl
             const int d = wide ? S.vt_off[x + 1] : int(c & 0xffffu);
             const int et = wide ? int(c) : int(c >> 16);
             S.vt_off[x + 1] = d;
-            et_b[x] = et;
+            if (!tight) et_b[x] = et;
             sv += d;
             se += et;
             if (d > caps.max_deg) flags |= ERR_CAPACITY;
@@ -863,7 +866,7 @@ __device__ bool run_cluster(const Team &tm, const DevMesh &m, const SmemPlan &pl
             }
         }
         int tot[4];
-        block_scan4(tm, sv, se, sn, su, S.scan, tot);
+        block_scan4(tm, sv, se, sn, su, S.scan, S.blk + kScanTotals, tot);
         vt_total = tot[0];
         et_total = tot[1];
         vv_total = tot[2];
@@ -872,13 +875,18 @@ __device__ bool run_cluster(const Team &tm, const DevMesh &m, const SmemPlan &pl
             (do_et && et_total > caps.max_etv))
             flags |= ERR_CAPACITY;
         for (int x = x0; x < x1; ++x) {
-            const int d = S.vt_off[x + 1], et = et_b[x];
-            if (d > 32) S.long_rows[atomicAdd(&flag[3], 1)] = uint16_t(x);
-            S.vt_off[x + 1] = sv + d;
-            if (!stride) cur[x] = (sv + x + 1) & ~1;
-            et_b[x] = se;
+            const int d = S.vt_off[x + 1];
+            if (tight) {
+                S.vt_off[x + 1] = sv;  // the cursor, which the fill moves to the row's end
+            } else {
+                const int et = et_b[x];
+                if (d > 32) S.long_rows[atomicAdd(&flag[kFlagLong], 1)] = uint16_t(x);
+                S.vt_off[x + 1] = sv + d;
+                if (!stride) cur[x] = (sv + x + 1) & ~1;
+                et_b[x] = se;
+                se += et;
+            }
             sv += d;
-            se += et;
             if (need_nb) {
                 const int n = S.c_vv[x], u = S.c_e[x];
                 S.c_vv[x] = sn | (n & int(0xff000000u));  // the bias stays on top
@@ -902,7 +910,8 @@ __device__ bool run_cluster(const Team &tm, const DevMesh &m, const SmemPlan &pl
 #pragma unroll
             for (int s = 0; s < 4; ++s) {
                 const uint32_t d = vtx(r, s) - uint32_t(lo);
-                if (d < nvo_u) fill[atomicAdd(&cur[d], 1)] = uint16_t(keyed ? 4 * i + s : i);
+                if (d < nvo_u)
+                    fill[atomicAdd(tight ? &S.vt_off[d + 1] : &cur[d], 1)] = uint16_t(keyed ? 4 * i + s : i);
             }
         }
         tm.sync();
@@ -914,8 +923,8 @@ __device__ bool run_cluster(const Team &tm, const DevMesh &m, const SmemPlan &pl
     // read the VV rows out of the bitmaps.  A sorted entry also gives the
     // position of its (tet, own vertex) in the row, kept for C3 and C5.
     {
-        const int half = (nvo + 1) >> 1, nlong = flag[3];
-        const int w_pair = (half + 31) >> 5, w_long = (nlong + 31) >> 5;
+        const int half = (nvo + 1) >> 1, nlong = flag[kFlagLong];
+        const int w_pair = tight ? 0 : (half + 31) >> 5, w_long = (nlong + 31) >> 5;
         const int w_emit = do_vv || do_et ? (nvo + 31) >> 5 : 0;
         for (int w = warp; w < w_pair + w_long + w_emit; w += NWARP) {
             if (w < w_pair) {
@@ -988,13 +997,14 @@ __device__ bool run_cluster(const Team &tm, const DevMesh &m, const SmemPlan &pl
             }
         }
         // stars of more than 64 tets: a warp each
-        if (caps.max_deg > 64)
-            for (int i = warp; i < nlong; i += NWARP) {
-                const int x = S.long_rows[i];
+        if (tight || caps.max_deg > 64)
+            for (int i = warp; i < (tight ? nvo : nlong); i += NWARP) {
+                const int x = tight ? i : S.long_rows[i];
                 const int o = S.vt_off[x], n = S.vt_off[x + 1] - o;
-                if (n <= 64) continue;
-                uint16_t *const v = fill + row_at(x);
+                if (n <= 64 && !tight) continue;
+                uint16_t *const v = fill + (tight ? o : row_at(x));
                 sort_row_warp(v, n, lane);
+                if (tight) continue;
                 for (int j = lane; j < n; j += 32) {
                     const uint32_t e = v[j];
                     S.vt_list[o + j] = uint16_t(keyed ? e >> 2 : e);
@@ -1066,7 +1076,7 @@ __device__ bool run_cluster(const Team &tm, const DevMesh &m, const SmemPlan &pl
     // the VV staging; masks of several words also reach the first ET entries,
     // which move to the vertex map (nvo <= nv_loc words)
     int32_t *const et_first = nch > 1 ? S.blk + kHdrWords : et_b;
-    if (nch > 1) {
+    if (nch > 1 && !tight) {
         for (int x = tid; x < nvo; x += NT) et_first[x] = et_b[x];
         tm.sync();
     }
@@ -1201,7 +1211,7 @@ __device__ bool run_cluster(const Team &tm, const DevMesh &m, const SmemPlan &pl
         if (nch == 1) links(IntC<1>{});
         else links(IntC<0>{});
         if (GEN && !PART && (flags & ERR_NONMANIFOLD)) {  // TT of this cluster takes the general pass (E')
-            flag[2] = 1;
+            flag[kFlagNonManifold] = 1;
             flags &= ~ERR_NONMANIFOLD;
         }
         if (flags) atomicOr(err, flags);
@@ -1272,8 +1282,25 @@ __device__ bool run_cluster(const Team &tm, const DevMesh &m, const SmemPlan &pl
                 }
             }
         };
-        if (nch == 1) rows_out(IntC<1>{});
-        else rows_out(IntC<0>{});
+        if (tight) {  // a vertex's edges by one thread, from sums over the masks
+            const int per = range_len(tm, nvo);
+            const int x0 = min(nvo, tid * per), x1 = min(nvo, x0 + per);
+            int n = 0, total;
+            for (int i = S.c_e[x0] * nch; i < S.c_e[x1] * nch; ++i) n += __popc(em[i]);
+            int run = block_scan_thread(tm, n, S.scan, &total);
+            bad = total != et_total;  // one distinct bit per entry
+            for (int x = x0; x < x1 && !bad; ++x)
+                for (int e = S.c_e[x]; e < S.c_e[x + 1]; ++e) {
+                    it->et_off[e] = run + b_et;
+                    for (int c = 0; c < nch; ++c)
+                        for (uint32_t mm = em[e * nch + c]; mm; mm &= mm - 1u)
+                            S.st_et[run++] = S.vt_list[S.vt_off[x] + 32 * c + __ffs(int(mm)) - 1];
+                }
+        } else if (nch == 1) {
+            rows_out(IntC<1>{});
+        } else {
+            rows_out(IntC<0>{});
+        }
         if (bad) {
             if (tid == 0) atomicOr(err, ERR_BAD_BLOCK);
             return true;
@@ -1350,12 +1377,12 @@ __device__ bool run_cluster(const Team &tm, const DevMesh &m, const SmemPlan &pl
             }
         }
         if (GEN && !PART && (flags & ERR_NONMANIFOLD)) {
-            flag[2] = 1;
+            flag[kFlagNonManifold] = 1;
             flags &= ~ERR_NONMANIFOLD;
         }
         if (flags) atomicOr(err, flags);
         tm.sync();
-        if (GEN && !PART && flag[2] != 0) {
+        if (GEN && !PART && flag[kFlagNonManifold] != 0) {
             tt_general<COUNT>(tm, S, rows, tmap, t_base, n_ext, n_own, n_vtets + h.n_halo, caps.max_tt, it,
                               sizes_out, err);
             return true;
@@ -1449,10 +1476,9 @@ __device__ bool run_cluster(const Team &tm, const DevMesh &m, const SmemPlan &pl
     return true;
 }
 
-// A work item: a whole cluster, or (id >= K) a part of a cut cluster.  GEN:
-// the whole-cluster instance carries the general TT pass (E'); the hot
-// shared-memory kernel leaves it out, and the clusters that need it (the
-// counting pass marks them) run from per-item bins.
+// A work item: a whole cluster, or (id >= K) a part of a cut cluster.  The
+// items that need GEN (non-manifold clusters, which the counting pass marks,
+// and tight plans) run from per-item bins.
 template <bool COUNT, bool SPILL, bool GEN, class Claim>
 __device__ __forceinline__ bool run_item(bool part, const DevMesh &m, const SmemPlan &plan, const Smem &S,
                                          int64_t blk_word, int64_t words, uint32_t mask, const WorkItem *it,
@@ -1576,7 +1602,7 @@ __global__ void __launch_bounds__(kMaxThreads) build_one_kernel(DevMesh m, SmemP
 constexpr int kMaxTeams = 15;  // named barriers 1..15
 constexpr int kMaxTeamBlock = 512;
 
-__global__ void __launch_bounds__(kMaxTeamBlock) build_kernel_team(DevMesh m, SmemPlan plan, const WorkItem *items,
+__global__ void __launch_bounds__(kMaxTeamBlock, 1) build_kernel_team(DevMesh m, SmemPlan plan, const WorkItem *items,
                                                                 const int32_t *order, int32_t n, int32_t *err,
                                                                 int32_t *ticket, int team_n) {
     extern __shared__ __align__(16) char smem[];
@@ -2024,7 +2050,44 @@ int64_t estimate_class(const ClusterStat &s, int threads) {
     return class_bytes(c, threads);
 }
 
-SmemPlan plan_smem(const Caps &c, int threads) {
+// The layout of kTight: no region beside those of class_bytes, none of them
+// larger, so that what the size class lets into shared memory fits there.
+static SmemPlan plan_tight(const Caps &c, int threads) {
+    SmemPlan p{};
+    p.threads = threads;
+    p.caps = c;
+    const int64_t nvo = c.nv_own;
+    p.W = std::max(1, (c.nv_nb + 31) / 32) | 1;
+    p.nch = std::max(1, (c.max_deg + 31) / 32);
+    p.mode = kTight | (c.max_deg > 256 ? kJpos16 : 0);
+    int64_t off = 0;
+    auto take = [&](int64_t bytes) {
+        const int64_t at = off;
+        off = a16(off + bytes);
+        return int32_t(std::min<int64_t>(at, INT32_MAX));
+    };
+    p.scan = take(4 * kScanWords);
+    p.blk = take(4 * int64_t(c.blk_words));
+    p.vt_off = take(4 * (nvo + 1));
+    p.fill = p.vt_list = take(2 * int64_t(c.n_vt));
+    p.c_vv = take(4 * (nvo + 1));
+    p.c_e = take(4 * (nvo + 1));
+    p.jpos = take((p.mode & kJpos16 ? 8 : 4) * int64_t(c.n_star));
+    // r2: VV staging, then the edge masks
+    p.et_b = p.long_rows = p.r2 = take(std::max(4 * int64_t(c.max_e) * p.nch, 2 * int64_t(c.max_vv)));
+    p.nbr = take(8 * int64_t(c.n_own));
+    // r1: bitmaps + rank prefixes | ET staging | face hash + TT counts + TT staging
+    const int64_t bm = a16(4 * nvo * p.W), hs = a16(4 * int64_t(c.hcap)), tc = a16(4 * (int64_t(c.n_own) + 1));
+    p.ex = p.r1 =
+        take(std::max(std::max(bm + nvo * p.W, 2 * int64_t(c.max_etv)), hs + tc + 2 * int64_t(c.max_tt)));
+    p.pre = int32_t(p.r1 + bm);
+    p.tcnt = int32_t(p.r1 + hs);
+    p.st_tt = int32_t(p.r1 + hs + tc);
+    p.total = off > INT32_MAX ? INT32_MAX : int32_t(off);
+    return p;
+}
+
+SmemPlan plan_smem(const Caps &c, int threads, bool shared) {
     SmemPlan p{};
     p.threads = threads;
     p.caps = c;
@@ -2044,7 +2107,7 @@ SmemPlan plan_smem(const Caps &c, int threads) {
             off = a16(off + bytes);
             return int32_t(std::min<int64_t>(at, INT32_MAX));
         };
-        p.scan = take(4 * scan_words(threads));
+        p.scan = take(4 * kScanWords);
         p.blk = take(4 * int64_t(c.blk_words));
         p.vt_off = take(4 * (nvo + 1));
         p.vt_list = take(2 * int64_t(c.n_vt));
@@ -2074,8 +2137,13 @@ SmemPlan plan_smem(const Caps &c, int threads) {
         p.tcnt = int32_t(p.r1 + hs);
         p.st_tt = int32_t(p.r1 + hs + tc);
         p.total = off > INT32_MAX ? INT32_MAX : int32_t(off);
-        if (!p.stride || off <= kPaddedFit) return p;
-        p.stride = 0;  // compact rows take less
+        if (p.stride && off > kPaddedFit) {
+            p.stride = 0;  // compact rows take less
+            continue;
+        }
+        if (!shared || off <= kCompactFit) return p;
+        const SmemPlan t = plan_tight(c, threads);
+        return t.total <= kCtaBytes ? t : p;
     }
 }
 

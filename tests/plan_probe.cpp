@@ -72,6 +72,25 @@ void probe_plans(gale_ctx *ctx, int32_t threads, int64_t *out) {
     }
 }
 
+// class, plan total and mode of n sets of capacities
+void probe_caps(const Caps *caps, int32_t n, int32_t threads, int64_t *out) {
+    for (int32_t i = 0; i < n; ++i, out += 3) {
+        const SmemPlan p = plan_smem(caps[i], threads);
+        out[0] = class_bytes(caps[i], threads);
+        out[1] = p.total;
+        out[2] = p.mode;
+    }
+}
+
+int32_t probe_caps_words() { return int32_t(sizeof(Caps) / sizeof(int32_t)); }
+
+// the constants plan_smem holds for a CTA's limit, and the device's
+void probe_limits(int64_t *out) {
+    out[0] = kCompactFit;
+    out[1] = kCtaBytes;
+    out[2] = dynamic_smem_limit();
+}
+
 // shared memory of one plan over the listed items (a size bin's)
 int64_t probe_merged(gale_ctx *ctx, const int32_t *ids, int32_t n, int32_t threads) {
     Caps m{};
