@@ -519,9 +519,14 @@ gale_status gale_get_bin_members(gale_ctx *ctx, int32_t *out);
  * working memory fits - and every CTA-per-SM count that fits, each timed
  * over reps launches (0 = 2) with CUDA events after one untimed launch; the
  * fastest pair is kept for the bin (gale_get_bins reports it) and captured
- * full builds are dropped so the next one captures the choice.  best_ms
- * (optional, max_bins entries): the chosen time per bin.  A later
- * gale_set_tuning call replaces the choice. */
+ * full builds are dropped so the next one captures the choice.  Where every
+ * item of the mesh has a CTA's place at once, one launch of all bins (512
+ * threads, each item under its own plan; what an untuned context does then,
+ * and for lists that short) is timed against them too, and if it is faster
+ * the bins take its block size; otherwise lists keep the bins' launches as
+ * well.  best_ms (optional, max_bins entries): the chosen time per bin, of
+ * the one launch where that was kept.  A later gale_set_tuning call replaces
+ * the choice. */
 gale_status gale_autotune(gale_ctx *ctx, uint32_t mask, int32_t reps, float *best_ms, int32_t max_bins);
 
 /* The stream of the context (cudaStream_t). */

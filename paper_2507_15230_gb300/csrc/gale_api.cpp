@@ -137,6 +137,7 @@ gale_status plan_bins(gale_ctx *ctx, bool with_sizes) {
     std::vector<int> tiers;
     for (int per = 4; per >= 1; --per) tiers.push_back(std::min(smem_sm / per - 1024 - kStaticMargin, smem_cta));
     ctx->bins.clear();
+    ctx->tuned_bins = false;
     ctx->bin_of.assign(NI, -1);
     size_t tier = 0;
     int cur_thr = 0;
@@ -362,9 +363,10 @@ SmemPlan serve_plan(gale_ctx *ctx, bool *fits, std::vector<uint8_t> *in_loop, st
 // threads 41.4, merged 32; 3 clusters of a Delaunay mesh in three bins 151
 // us a call, merged 62.  The line
 // lies where the items no longer all fit.  A block size or occupancy set by
-// the caller, teams and global-scratch bins keep their bins' launches.
+// the caller, bins that gale_autotune kept, teams and global-scratch bins
+// keep their bins' launches.
 bool merged_launch(const gale_ctx *ctx, const int32_t *items, int32_t n, SmemPlan *env) {
-    if (n < 1 || ctx->threads_override || ctx->ctas_override || n > ctx->merged_per_sm * ctx->sm_count) return false;
+    if (n < 1 || ctx->threads_override || ctx->ctas_override || ctx->tuned_bins || n > ctx->merged_per_sm * ctx->sm_count) return false;
     int top = 0, first = -1;
     bool several = false;
     for (int32_t i = 0; i < n; ++i) {
@@ -662,6 +664,48 @@ cudaError_t run_bins(gale_ctx *ctx, const gale::DevMesh &dm, const WorkItem *ite
         if (e == cudaSuccess) e = j;
     }
     return e;
+}
+
+// The batched build of every cluster as an executable graph.
+gale_status capture_full(gale_ctx *ctx, uint32_t mask, cudaGraphExec_t *g, int64_t *launches) {
+    const gale::DevMesh dm = dev_mesh(ctx);
+    const int32_t ni = int32_t(ctx->all_items.size());
+    gale::SmemPlan env;
+    const bool merged = gale::merged_launch(ctx, ctx->all_items.data(), ni, &env);
+    std::vector<BinRun> runs;
+    for (size_t b = 0; !merged && b < ctx->bins.size(); ++b)
+        if (!ctx->bins[b].cut)  // a cut bin's clusters' parts are in other bins
+            runs.push_back({b, ctx->d_order_all + ctx->order_all_off[b], int32_t(ctx->bins[b].clusters.size())});
+    if (runs.size() > 1)  // not while capturing
+        CUDA_TRY(ensure_bin_streams(ctx, std::min<size_t>(runs.size() - 1, kBinStreams)));
+    CUDA_TRY(cudaStreamBeginCapture(ctx->stream, cudaStreamCaptureModeThreadLocal));
+    cudaGraph_t graph;
+    int nl = 0;
+    int64_t builds = 0;
+    int rc = gale::launch_bases(dm, ctx->hm.NP ? ctx->d_all_items : nullptr, ni, ctx->d_sizes, mask,
+                                ctx->d_arrays_base + mask, ctx->d_items, ctx->d_totals, ctx->d_bsum, ctx->d_tickets,
+                                int(ctx->bins.size()), ctx->stream, &nl);
+    if (rc == 0 && merged) {
+        builds = 1;
+        rc = gale::launch_build(dm, env, ctx->d_items, nullptr, ni, ctx->d_err, ctx->d_tickets, ni, ctx->stream,
+                                nullptr, ctx->d_plans, 0, false);
+    } else if (rc == 0) {
+        rc = int(run_bins(ctx, dm, ctx->d_items, std::move(runs), &builds));
+    }
+    *launches = nl + builds;
+    cudaError_t ce = cudaStreamEndCapture(ctx->stream, &graph);
+    if (ce != cudaSuccess) return cuda_fail(rc != 0 ? cudaError_t(rc) : ce, "capturing the batched build");
+    if (rc != 0) {
+        cudaGraphDestroy(graph);
+        return cuda_fail(cudaError_t(rc), "capturing the batched build");
+    }
+    ce = cudaGraphInstantiate(g, graph, 0);
+    cudaGraphDestroy(graph);
+    if (ce != cudaSuccess) {
+        *g = nullptr;
+        return cuda_fail(ce, "cudaGraphInstantiate");
+    }
+    return GALE_OK;
 }
 
 gale_status ensure_bulk(gale_ctx *ctx, const int64_t *need) {
@@ -1046,39 +1090,8 @@ gale_status gale_build_clusters(gale_ctx *ctx, const int32_t *ids, int32_t n, ui
     if (mode == GALE_MODE_BATCHED && all) {
         cudaGraphExec_t &g = ctx->graphs[mask];
         if (!g) {
-            cudaGraph_t graph;
-            const int32_t ni = int32_t(ctx->all_items.size());
-            gale::SmemPlan env;
-            const bool merged = gale::merged_launch(ctx, ctx->all_items.data(), ni, &env);
-            std::vector<BinRun> runs;
-            for (size_t b = 0; !merged && b < ctx->bins.size(); ++b)
-                if (!ctx->bins[b].cut)  // a cut bin's clusters' parts are in other bins
-                    runs.push_back({b, ctx->d_order_all + ctx->order_all_off[b], int32_t(ctx->bins[b].clusters.size())});
-            if (runs.size() > 1)  // not while capturing
-                CUDA_TRY(ensure_bin_streams(ctx, std::min<size_t>(runs.size() - 1, kBinStreams)));
-            CUDA_TRY(cudaStreamBeginCapture(ctx->stream, cudaStreamCaptureModeThreadLocal));
-            int nl = 0;
-            int64_t builds = 0;
-            int rc = gale::launch_bases(dm, ctx->hm.NP ? ctx->d_all_items : nullptr, ni, ctx->d_sizes, mask, base,
-                                        ctx->d_items, ctx->d_totals, ctx->d_bsum, ctx->d_tickets,
-                                        int(ctx->bins.size()), ctx->stream, &nl);
-            if (rc == 0 && merged) {
-                builds = 1;
-                rc = gale::launch_build(dm, env, ctx->d_items, nullptr, ni, ctx->d_err, ctx->d_tickets, ni, ctx->stream,
-                                        nullptr, ctx->d_plans, 0, false);
-            } else if (rc == 0) {
-                rc = int(run_bins(ctx, dm, ctx->d_items, std::move(runs), &builds));
-            }
-            ctx->graph_launches[mask] = nl + builds;
-            cudaError_t ce = cudaStreamEndCapture(ctx->stream, &graph);
-            if (rc != 0) return cuda_fail(cudaError_t(rc), "capturing the batched build");
-            if (ce != cudaSuccess) return cuda_fail(ce, "cudaStreamEndCapture");
-            ce = cudaGraphInstantiate(&g, graph, 0);
-            cudaGraphDestroy(graph);
-            if (ce != cudaSuccess) {
-                g = nullptr;
-                return cuda_fail(ce, "cudaGraphInstantiate");
-            }
+            const gale_status st = capture_full(ctx, mask, &g, &ctx->graph_launches[mask]);
+            if (st != GALE_OK) return st;
         }
         CUDA_TRY(cudaGraphLaunch(g, ctx->stream));
         launches = ctx->graph_launches[mask];
@@ -1673,8 +1686,6 @@ gale_status gale_autotune(gale_ctx *ctx, uint32_t mask, int32_t reps, float *bes
         }
         if (best_ms && int32_t(b) < max_bins) best_ms[b] = best;
     }
-    cudaEventDestroy(e0);
-    cudaEventDestroy(e1);
     int max_total = 0;
     for (auto &bin : ctx->bins)
         if (!bin.spill) max_total = std::max(max_total, bin.plan.total * std::max(1, bin.teams));
@@ -1684,8 +1695,46 @@ gale_status gale_autotune(gale_ctx *ctx, uint32_t mask, int32_t reps, float *bes
             cudaGraphExecDestroy(g);
             g = nullptr;
         }
-    st = check_device_error(ctx);
-    return st;
+    // A mesh whose items all have a CTA's place at once: the bins as tuned
+    // against one launch of all of them, each as a replayed graph.  Where the
+    // one launch is the faster, the bins take its block size.
+    ctx->tuned_bins = false;
+    gale::SmemPlan env;
+    if (gale::merged_launch(ctx, ctx->all_items.data(), int32_t(ctx->all_items.size()), &env)) {
+        float ms[2] = {};
+        for (int one = 0; st == GALE_OK && one < 2; ++one) {
+            ctx->tuned_bins = one == 0;
+            cudaGraphExec_t g = nullptr;
+            int64_t nl = 0;
+            st = capture_full(ctx, mask, &g, &nl);
+            if (st != GALE_OK) break;
+            const int n = std::max(reps, 8);  // of some tens of microseconds each
+            cudaError_t e = cudaGraphLaunch(g, ctx->stream);
+            if (e == cudaSuccess) e = cudaEventRecord(e0, ctx->stream);
+            for (int r = 0; e == cudaSuccess && r < n; ++r) e = cudaGraphLaunch(g, ctx->stream);
+            if (e == cudaSuccess) e = cudaEventRecord(e1, ctx->stream);
+            if (e == cudaSuccess) e = cudaEventSynchronize(e1);
+            if (e == cudaSuccess) e = cudaEventElapsedTime(&ms[one], e0, e1);
+            cudaGraphExecDestroy(g);
+            if (e != cudaSuccess) st = cuda_fail(e, "timing the batched build");
+            ms[one] /= float(n);
+        }
+        ctx->tuned_bins = st == GALE_OK && ms[0] <= ms[1];
+        for (size_t b = 0; st == GALE_OK && !ctx->tuned_bins && b < ctx->bins.size(); ++b) {
+            gale::Bin &bin = ctx->bins[b];
+            if (bin.cut) continue;
+            bin.plan.threads = env.threads;  // (no layout depends on it)
+            bin.ctas_per_sm = gale::max_ctas_per_sm(bin.plan, false, bin.per_item);
+            bin.grid = std::max(1, std::min<int>(int(bin.clusters.size()), bin.ctas_per_sm * ctx->sm_count));
+            if (best_ms && int32_t(b) < max_bins) best_ms[b] = ms[1];
+        }
+    } else {
+        ctx->tuned_bins = true;
+    }
+    cudaEventDestroy(e0);
+    cudaEventDestroy(e1);
+    const gale_status dst = check_device_error(ctx);
+    return st != GALE_OK ? st : dst;
 }
 
 gale_status gale_get_bins(gale_ctx *ctx, int32_t *out, int32_t max_bins, int32_t *nbins) {

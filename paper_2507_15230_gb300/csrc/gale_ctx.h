@@ -90,6 +90,7 @@ struct gale_ctx {
     std::vector<int64_t> order_all_off; // [nbins+1] offsets into d_order_all
     int threads_override = 0;  // 0: chosen from the cluster's tet count
     int ctas_override = 0;
+    bool tuned_bins = false;  // gale_autotune kept the bins' own launches (not the merged one)
     int sm_count = 0;
     int smem_sm = 0;        // shared memory of an SM
     int merged_per_sm = 0;  // CTAs of a merged launch an SM holds by threads and registers
