@@ -97,17 +97,13 @@ gale_status plan_bins(gale_ctx *ctx, bool with_sizes) {
     const int32_t K = ctx->hm.K;
     const int32_t NI = K + ctx->hm.NP;
     // dynamic shared memory a CTA may plan for: the opt-in limit less the
-    // kernels' static shared memory
+    // kernels' static shared memory.  (The tiers leave 512 bytes of the SM's
+    // share: the hot kernel has 272.)
     constexpr int kStaticMargin = 512;
     const int smem_cta = gale::dynamic_smem_limit();
     int smem_sm = 0;
     cudaDeviceGetAttribute(&smem_sm, cudaDevAttrMaxSharedMemoryPerMultiprocessor, ctx->device);
-    ctx->smem_sm = smem_sm;
-    {
-        gale::SmemPlan p{};
-        p.threads = kMergedThreads;
-        ctx->merged_per_sm = gale::max_ctas_per_sm(p, false, true);
-    }
+    for (int c = 0; c < 4; ++c) ctx->merged_fit[c] = gale::per_item_fit(c + 1, kMergedThreads);
     auto caps_k = [&](int32_t k) {
         return gale::caps_of(ctx->hm.stats[k], with_sizes ? ctx->sizes.data() + size_t(5) * k : nullptr);
     };
@@ -353,6 +349,14 @@ SmemPlan serve_plan(gale_ctx *ctx, bool *fits, std::vector<uint8_t> *in_loop, st
     if (in_loop) *in_loop = sel;
     return env;
 }
+// CTAs of a merged launch that an SM holds when each takes `total` bytes of
+// dynamic shared memory.
+int merged_ctas(const gale_ctx *ctx, int total) {
+    int c = 0;
+    while (c < 4 && ctx->merged_fit[c] >= total) ++c;
+    return c;
+}
+
 // Short lists.  Size bins are launched one after another or side by side,
 // each with its own block size and occupancy, which pays when a bin fills the
 // GPU.  Where every listed item has a CTA's place at once, one launch of
@@ -366,7 +370,9 @@ SmemPlan serve_plan(gale_ctx *ctx, bool *fits, std::vector<uint8_t> *in_loop, st
 // the caller, bins that gale_autotune kept, teams and global-scratch bins
 // keep their bins' launches.
 bool merged_launch(const gale_ctx *ctx, const int32_t *items, int32_t n, SmemPlan *env) {
-    if (n < 1 || ctx->threads_override || ctx->ctas_override || ctx->tuned_bins || n > ctx->merged_per_sm * ctx->sm_count) return false;
+    if (n < 1 || ctx->threads_override || ctx->ctas_override || ctx->tuned_bins ||
+        n > merged_ctas(ctx, 0) * ctx->sm_count)
+        return false;
     int top = 0, first = -1;
     bool several = false;
     for (int32_t i = 0; i < n; ++i) {
@@ -378,8 +384,7 @@ bool merged_launch(const gale_ctx *ctx, const int32_t *items, int32_t n, SmemPla
         first = b;
         top = std::max(top, ctx->h_plans[items[i]].total);
     }
-    const int per_sm = std::min(ctx->merged_per_sm, ctx->smem_sm / (top + 1024 + 512));
-    if (!several || n > per_sm * ctx->sm_count) return false;
+    if (!several || n > merged_ctas(ctx, top) * ctx->sm_count) return false;
     *env = SmemPlan{};
     env->threads = kMergedThreads;
     env->total = top;

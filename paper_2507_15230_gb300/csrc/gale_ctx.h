@@ -92,8 +92,8 @@ struct gale_ctx {
     int ctas_override = 0;
     bool tuned_bins = false;  // gale_autotune kept the bins' own launches (not the merged one)
     int sm_count = 0;
-    int smem_sm = 0;        // shared memory of an SM
-    int merged_per_sm = 0;  // CTAs of a merged launch an SM holds by threads and registers
+    int merged_fit[4] = {};  // dynamic shared memory a CTA of a merged launch may take with 1 to 4 of them on
+                             // an SM (-1: so many do not fit by threads and registers)
 
     // bulk output arrays
     int32_t *bulk[10] = {};
@@ -147,6 +147,7 @@ namespace gale {
 gale_status copy_to_host(gale_ctx *ctx, void *dst, const void *src, size_t bytes);
 // Lengths of the ten output arrays of cluster k under mask (gale_api.cpp).
 void item_lengths(const gale_ctx *ctx, int32_t k, uint32_t mask, int64_t *L);
+int merged_ctas(const gale_ctx *ctx, int total);
 // Whether these work items are built by one merged launch (gale_api.cpp):
 // *env gets its block size and shared memory.
 bool merged_launch(const gale_ctx *ctx, const int32_t *items, int32_t n, SmemPlan *env);

@@ -308,6 +308,9 @@ int kernel_smem_limit();
 int max_ctas_per_sm(const SmemPlan &plan, bool spill, bool per_item = false);
 // CTAs per SM of a team launch (0 if it cannot launch)
 int max_ctas_per_sm_teams(const SmemPlan &plan, int teams);
+// dynamic shared memory a CTA of the per-item build kernel may take with
+// `ctas` of them on an SM; -1 if so many do not fit at this block size
+int per_item_fit(int ctas, int threads);
 // Sets the dynamic shared memory limit of the cluster kernels to smem
 // (clamped to dynamic_smem_limit()); false if the runtime refused.
 bool prepare_kernels(int smem);

@@ -2220,6 +2220,23 @@ int max_ctas_per_sm(const SmemPlan &plan, bool spill, bool per_item) {
     return a < b ? a : b;
 }
 
+int per_item_fit(int ctas, int threads) {
+    SmemPlan p{};
+    p.threads = threads;
+    cudaFuncAttributes a;
+    int dev = 0, sm = 0, reserved = 0;
+    cudaGetDevice(&dev);
+    if (max_ctas_per_sm(p, false, true) < ctas || cudaFuncGetAttributes(&a, build_kernel_pi) != cudaSuccess ||
+        cudaDeviceGetAttribute(&sm, cudaDevAttrMaxSharedMemoryPerMultiprocessor, dev) != cudaSuccess ||
+        cudaDeviceGetAttribute(&reserved, cudaDevAttrReservedSharedMemoryPerBlock, dev) != cudaSuccess) {
+        cudaGetLastError();
+        return -1;
+    }
+    // (the occupancy API answers within the limit granted so far; a CTA's
+    // share is whole 128-byte units)
+    return std::min((sm / ctas & ~127) - reserved, kernel_smem_limit()) - int(a.sharedSizeBytes);
+}
+
 int max_ctas_per_sm_teams(const SmemPlan &plan, int teams) {
     if (teams < 1 || teams > kMaxTeams || plan.threads % 32 || plan.threads * teams > kMaxTeamBlock) return 0;
     int a = 0;

@@ -91,6 +91,16 @@ void probe_limits(int64_t *out) {
     out[2] = dynamic_smem_limit();
 }
 
+// CTAs an SM holds at `total` bytes: as merged launches plan, and the device's
+void probe_merged_ctas(gale_ctx *ctx, int32_t total, int32_t *out) {
+    prepare_kernels(dynamic_smem_limit());
+    SmemPlan p{};
+    p.threads = 512;
+    p.total = total;
+    out[0] = merged_ctas(ctx, total);
+    out[1] = max_ctas_per_sm(p, false, true);
+}
+
 // shared memory of one plan over the listed items (a size bin's)
 int64_t probe_merged(gale_ctx *ctx, const int32_t *ids, int32_t n, int32_t threads) {
     Caps m{};

@@ -4,6 +4,7 @@ A size bin's plan is made from the maxima over its members, and that plan
 can be smaller than a member's own: one longer star takes the padded rows
 away from the whole bin.  The launch of a short list asks for the largest
 member's plan, so that is what the kernels' limit has to allow."""
+import ctypes
 import os
 import subprocess
 import sys
@@ -15,7 +16,7 @@ import gen
 import oracle
 import paper_2507_15230_gb300 as gale
 from parity_util import assert_bulk_equal, expected_bulk
-from plan_util import item_plans, merged_total
+from plan_util import item_plans, merged_total, probe
 
 ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
 
@@ -85,3 +86,16 @@ def test_list_with_the_largest_member_in_a_fresh_process():
                        env=dict(os.environ, PYTHONPATH=os.pathsep.join([ROOT, os.path.join(ROOT, "tests")])),
                        capture_output=True, text=True, timeout=300)
     assert r.returncode == 0, r.stderr[-3000:]
+
+
+@pytest.mark.gpu
+def test_planned_occupancy_is_the_devices():
+    """The kernel's static shared memory counts: two CTAs of 115,200 bytes
+    each do not fit an SM beside it."""
+    out = (ctypes.c_int32 * 2)()
+    with gale.Context.load(gen.small_grid(with_field=False), device=0) as ctx:
+        for total in (0, 16, 57_344, 74_000, 113_000, *range(114_000, 116_000, 16), 150_000, 230_000, 230_816):
+            probe().probe_merged_ctas(ctx._h, total, out)
+            assert out[0] == out[1] >= 1, total
+        probe().probe_merged_ctas(ctx._h, 115_200, out)
+        assert out[0] == 1
