@@ -1090,32 +1090,34 @@ gale_status run_pass(gale_ctx *ctx, uint32_t which, const EnumView &ev, int32_t 
     const bool vf_gather = wVF && cb.sorted_ids, vf_scatter = wVF && !cb.sorted_ids;
     const bool wVE = (which & GALE_CB_VE) || vf_gather, wEF = (which & GALE_CB_EF) || vf_gather;
     const bool ft_gen = wFT && cb.ft_general;
-    // scratch: counters (zeroed), then ranks and lookups
-    auto al = [](int64_t x) { return (x + 3) & ~int64_t(3); };
-    const int64_t n_ctr = 2 * al(hm.nv) + 2 * al(nE);
-    const int64_t n_scr = n_ctr + al(hm.nv) + 3 * al(nE) + 4 * al(nF) + 2 * al(nF);
+    // scratch of the relations that are built: counters (zeroed), then ranks
+    // and lookups.  FT comes last, and its slots take the place of the
+    // triangles' lookups.
+    int64_t n_scr = 0;
+    auto take = [&](bool wanted, int64_t n) {
+        const int64_t at = n_scr;
+        if (wanted) n_scr += (n + 3) & ~int64_t(3);
+        return at;
+    };
+    const int64_t o_ve_n = take(wVE, hm.nv), o_vf_n = take(wVF, hm.nv);
+    const int64_t o_ef_lo = take(wEF, nE), o_ef_mid = take(wEF, nE);
+    const int64_t n_ctr = n_scr;
+    const int64_t o_vf_fill = take(vf_scatter, hm.nv), o_ve_rank = take(wVE, nE), o_ef_tail = take(vf_gather, 2 * nE);
+    const int64_t o_tri = take(wEF || wFT, std::max<int64_t>({2, wEF ? 4 * nF : 0, wFT && !ft_gen ? 2 * nF : 0}));
+    const int64_t n_cnt = std::max({wVE || wVF ? hm.nv : 1, wEF ? nE : 1, ft_gen ? nF : 1});
     if (!grow(ctx, cb.scratch, cb.scratch_cap, std::max<int64_t>(n_scr, 4)) ||
-        !grow(ctx, cb.cnt, cb.cnt_cap, std::max<int64_t>({hm.nv, nE, nF, int64_t(1)})))
+        !grow(ctx, cb.cnt, cb.cnt_cap, n_cnt))
         return fail(GALE_ENOMEM, "device allocation of coboundary scratch failed");
     Scatter sc{};
-    {
-        int32_t *q = cb.scratch;
-        auto take = [&](int64_t n) {
-            int32_t *r = q;
-            q += n;
-            return r;
-        };
-        sc.ve_n = take(al(hm.nv));
-        sc.vf_n = take(al(hm.nv));
-        sc.ef_lo = take(al(nE));
-        sc.ef_mid = take(al(nE));
-        sc.vf_fill = take(al(hm.nv));
-        sc.ve_rank = take(al(nE));
-        sc.ef_tail = reinterpret_cast<int2 *>(take(2 * al(nE)));
-        sc.tri = reinterpret_cast<int4 *>(take(4 * al(nF)));
-        sc.ft_slot = reinterpret_cast<int2 *>(take(2 * al(nF)));
-        if (!vf_gather) sc.ef_tail = nullptr;
-    }
+    sc.ve_n = cb.scratch + o_ve_n;
+    sc.vf_n = cb.scratch + o_vf_n;
+    sc.ef_lo = cb.scratch + o_ef_lo;
+    sc.ef_mid = cb.scratch + o_ef_mid;
+    sc.vf_fill = cb.scratch + o_vf_fill;
+    sc.ve_rank = cb.scratch + o_ve_rank;
+    sc.ef_tail = vf_gather ? reinterpret_cast<int2 *>(cb.scratch + o_ef_tail) : nullptr;
+    sc.tri = reinterpret_cast<int4 *>(cb.scratch + o_tri);
+    sc.ft_slot = reinterpret_cast<int2 *>(cb.scratch + o_tri);
     sc.cnt = cb.cnt;
     if (cudaMemsetAsync(cb.scratch, 0, sizeof(int32_t) * size_t(n_ctr), s) != cudaSuccess)
         return fail(GALE_ECUDA, "cudaMemsetAsync");
