@@ -85,6 +85,24 @@ int threads_for(const gale_ctx *ctx, const gale::ClusterStat &s) {
 
 constexpr int kMergedThreads = 512;
 
+constexpr int kBinStreams = 5;  // beside the context's own
+
+cudaError_t ensure_bin_streams(gale_ctx *ctx, size_t ns) {
+    while (ctx->bin_streams.size() < ns) {
+        cudaStream_t st;
+        const cudaError_t e = cudaStreamCreateWithFlags(&st, cudaStreamNonBlocking);
+        if (e != cudaSuccess) return e;
+        ctx->bin_streams.push_back(st);
+    }
+    while (ctx->bin_events.size() < ns + 1) {
+        cudaEvent_t ev;
+        const cudaError_t e = cudaEventCreateWithFlags(&ev, cudaEventDisableTiming);
+        if (e != cudaSuccess) return e;
+        ctx->bin_events.push_back(ev);
+    }
+    return cudaSuccess;
+}
+
 // Size bins: work items (clusters, then the parts of cut clusters) sorted by
 // shared-memory need, cut where the merged plan would cross the next
 // occupancy tier (4, 3, 2, 1 CTAs per SM).  Items whose plan exceeds the
@@ -283,6 +301,14 @@ gale_status plan_bins(gale_ctx *ctx, bool with_sizes) {
         ctx->spill_bytes = ctx->d_spill ? spill_need : 0;
         if (!ctx->d_spill) return fail(GALE_ENOMEM, "device allocation of the large-cluster scratch failed");
     }
+    // the streams that several bins' launches fork to: here, as the first
+    // build is 40 us slower when it makes them (a list of an 80^3 grid: 385
+    // us, 346 before builds forked)
+    size_t nb = 0;
+    for (auto &b : ctx->bins) nb += !b.cut;
+    gale::SmemPlan env;
+    if (with_sizes && nb > 1 && !gale::merged_launch(ctx, ctx->all_items.data(), int32_t(ctx->all_items.size()), &env))
+        CUDA_TRY(ensure_bin_streams(ctx, std::min<size_t>(nb - 1, kBinStreams)));
     return GALE_OK;
 }
 
@@ -610,24 +636,6 @@ struct BinRun {
     const int32_t *order;
     int32_t n;
 };
-
-constexpr int kBinStreams = 5;  // beside the context's own
-
-cudaError_t ensure_bin_streams(gale_ctx *ctx, size_t ns) {
-    while (ctx->bin_streams.size() < ns) {
-        cudaStream_t st;
-        const cudaError_t e = cudaStreamCreateWithFlags(&st, cudaStreamNonBlocking);
-        if (e != cudaSuccess) return e;
-        ctx->bin_streams.push_back(st);
-    }
-    while (ctx->bin_events.size() < ns + 1) {
-        cudaEvent_t ev;
-        const cudaError_t e = cudaEventCreateWithFlags(&ev, cudaEventDisableTiming);
-        if (e != cudaSuccess) return e;
-        ctx->bin_events.push_back(ev);
-    }
-    return cudaSuccess;
-}
 
 // The bins' launches, after the placement pass on the context stream (which
 // zeroed the tickets).  Several bins run side by side: forked to streams of

@@ -101,6 +101,8 @@ void probe_merged_ctas(gale_ctx *ctx, int32_t total, int32_t *out) {
     out[1] = max_ctas_per_sm(p, false, true);
 }
 
+int32_t probe_bin_streams(gale_ctx *ctx) { return int32_t(ctx->bin_streams.size()); }
+
 // shared memory of one plan over the listed items (a size bin's)
 int64_t probe_merged(gale_ctx *ctx, const int32_t *ids, int32_t n, int32_t threads) {
     Caps m{};
