@@ -12,7 +12,7 @@ pytestmark = pytest.mark.gpu
 
 
 def launches(ctx):
-    return gale.load_library().gale_last_launch_count(ctx._h)
+    return ctx.last_launch_count()
 
 
 @pytest.mark.parametrize("kind", ["grid16", "grid24", "delaunay4000", "delaunay12000"])
