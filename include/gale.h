@@ -476,8 +476,8 @@ typedef struct {
 gale_status gale_build_coboundary(gale_ctx *ctx, uint32_t which, gale_coboundary *out);
 
 /* Tuning: threads per block of the producer kernels (a multiple of 32 in
- * [64, 1024]; 0 = one thread per own vertex of the largest cluster of each
- * size bin) and CTAs per SM of the persistent grid (0 = as many as fit). */
+ * [64, 1024]; 0 = about one thread per five tets of a cluster, a power of two
+ * from 64 to 512) and CTAs per SM of the persistent grid (0 = as many as fit). */
 gale_status gale_set_tuning(gale_ctx *ctx, int32_t threads, int32_t ctas_per_sm);
 
 /* Several small clusters per CTA (no counterpart in the paper, which runs a

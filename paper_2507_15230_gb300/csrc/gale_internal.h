@@ -171,7 +171,7 @@ struct SmemPlan {
     int32_t W;          // row stride (words, odd) of the neighbour bitmaps
     int32_t nch;        // 32-tet chunks of the longest VT row
     int32_t stride;     // row stride of the padded rows (uint16s; 0: compact rows)
-    int32_t fill;       // the rows in arrival order (inside r2 and nbr)
+    int32_t fill;       // the rows in arrival order (inside r2 and nbr; kTight: vt_list itself)
     int32_t mode;       // kKeyed: the rows' entries carry the vertex's slot in the tet;
                         // kJpos16: VT rows may exceed 256 entries, positions are 16-bit;
                         // kTight: the smallest layout (kernels that carry the rare forms)

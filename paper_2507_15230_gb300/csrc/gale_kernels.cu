@@ -40,9 +40,9 @@
 //  E. TT rows from the four face links, sorted by canonical id.  A face with
 //     a second partner (a triangle in three or more tets) marks the cluster
 //     instead, whose rows then come from E', a general pass over the block
-//     (compiled into every kernel but the hot shared-memory one: the
-//     counting pass reports such clusters and the host runs them from
-//     per-item bins).  Parts of cut clusters report it as an error.
+//     (compiled into every kernel but the hot shared-memory one, as is the
+//     tight layout: the host runs clusters that need either from per-item
+//     bins; the counting pass reports the non-manifold ones).  Parts of cut clusters report it as an error.
 //
 // The counting mode runs the same passes without writes and returns the
 // exact sizes the host uses to place outputs and to admit cache entries.
@@ -356,7 +356,8 @@ struct IntC {
 
 // stars larger than this count their tets and ET entries in two words
 constexpr int32_t kMaxPacked = 21845;
-constexpr int kOffMask = 0xffffff;  // VV offsets (at most 6 x 65534) under the 8-bit bias
+// VV offsets (a tet adds up to 12 entries: 12 x 65,534 < 2^24) under the 8-bit bias
+constexpr int kOffMask = 0xffffff;
 
 __device__ __forceinline__ void cmpx_u16x2(uint32_t &a, uint32_t &b) {
     uint32_t lo, hi;
