@@ -1492,7 +1492,7 @@ gale_status gale_set_teams(gale_ctx *ctx, int32_t team_threads, int32_t teams) {
             b.teams = 0;
             continue;
         }
-        const gale::SmemPlan p = gale::plan_smem(b.plan.caps, team_threads, false);
+        gale::SmemPlan p = gale::plan_smem(b.plan.caps, team_threads, false);
         if (int64_t(p.total) * teams > smem_limit) continue;
         max_total = std::max(max_total, p.total * teams);
         if (!gale::prepare_kernels(max_total)) return fail(GALE_ECUDA, "setting the kernels' shared memory limit failed");
@@ -1650,7 +1650,7 @@ gale_status gale_autotune(gale_ctx *ctx, uint32_t mask, int32_t reps, float *bes
             for (int T : {32, 64, 128})
                 for (int tm : {2, 4, 8}) {
                     if (T * tm > 512) continue;
-                    const gale::SmemPlan plan = gale::plan_smem(bin.plan.caps, T, false);
+                    gale::SmemPlan plan = gale::plan_smem(bin.plan.caps, T, false);
                     if (int64_t(plan.total) * tm > smem_limit) continue;
                     const int per = gale::max_ctas_per_sm_teams(plan, tm);
                     if (per < 1) continue;

@@ -165,7 +165,7 @@ struct Caps {
 //       the boundary-face hash, the TT counts and the TT staging.
 // Tight plans (kTight) fill and sort VT's rows in place and keep neither the
 // first ET entries nor long rows.
-constexpr int32_t kKeyed = 1, kJpos16 = 2, kTight = 4;
+constexpr int32_t kKeyed = 1, kJpos16 = 2, kTight = 4, kLeanTeam = 8;
 struct SmemPlan {
     int32_t threads;
     int32_t W;          // row stride (words, odd) of the neighbour bitmaps
@@ -174,7 +174,8 @@ struct SmemPlan {
     int32_t fill;       // the rows in arrival order (inside r2 and nbr; kTight: vt_list itself)
     int32_t mode;       // kKeyed: the rows' entries carry the vertex's slot in the tet;
                         // kJpos16: VT rows may exceed 256 entries, positions are 16-bit;
-                        // kTight: the smallest layout (kernels that carry the rare forms)
+                        // kTight: the smallest layout (kernels that carry the rare forms);
+                        // kLeanTeam: team launches take the instance of fewer registers
     int32_t scan;       // scan scratch
     int32_t blk;        // int32[blk_words] the cluster's block (bulk copy)
     int32_t vt_off;     // int32[nv_own+1]
@@ -307,7 +308,7 @@ int serve_ctas_per_sm(const SmemPlan &plan);
 int kernel_smem_limit();
 int max_ctas_per_sm(const SmemPlan &plan, bool spill, bool per_item = false);
 // CTAs per SM of a team launch (0 if it cannot launch)
-int max_ctas_per_sm_teams(const SmemPlan &plan, int teams);
+int max_ctas_per_sm_teams(SmemPlan &plan, int teams);  // (sets kLeanTeam)
 // dynamic shared memory a CTA of the per-item build kernel may take with
 // `ctas` of them on an SM; -1 if so many do not fit at this block size
 int per_item_fit(int ctas, int threads);

@@ -1599,13 +1599,24 @@ __global__ void __launch_bounds__(kMaxThreads) build_one_kernel(DevMesh m, SmemP
 // ticket on its own and builds each in its own slice of the dynamic shared
 // memory, with a named barrier and a bulk-copy barrier of its own, so a
 // small cluster's barriers involve only its team.
+//
+// Two instances.  Left alone the compiler takes 95 registers and spills none,
+// which is the faster code, but one CTA of 512 threads then fills an SM's
+// registers; at 64 (LEAN) two fit.  With as many CTAs on an SM the first is 4
+// to 8 % faster, with half as many the second is: 64^3 grid of 64-vertex
+// leaves, teams of 128 x 4 260 -> 199 us a build (one CTA an SM against two),
+// 128 x 2 254 -> 188 (two against four), 64 x 2 195 against 205 (four of
+// either).  At two against three it goes either way (64 x 4 205 against 215;
+// 128-vertex leaves, 128 x 2 181 against 158).  So the plan takes the second
+// where it holds twice the CTAs (kLeanTeam, max_ctas_per_sm_teams).
 // ---------------------------------------------------------------------------
 constexpr int kMaxTeams = 15;  // named barriers 1..15
 constexpr int kMaxTeamBlock = 512;
 
-__global__ void __launch_bounds__(kMaxTeamBlock, 1) build_kernel_team(DevMesh m, SmemPlan plan, const WorkItem *items,
-                                                                const int32_t *order, int32_t n, int32_t *err,
-                                                                int32_t *ticket, int team_n) {
+template <bool LEAN>
+__global__ void __launch_bounds__(kMaxTeamBlock, LEAN ? 2 : 1)
+    build_kernel_team(DevMesh m, SmemPlan plan, const WorkItem *items, const int32_t *order, int32_t n, int32_t *err,
+                      int32_t *ticket, int team_n) {
     extern __shared__ __align__(16) char smem[];
     __shared__ int32_t s_idx[kMaxTeams];
     __shared__ WorkItem s_item[kMaxTeams];
@@ -2175,7 +2186,10 @@ int dynamic_smem_limit() {
     if (cudaFuncGetAttributes(&a, serve_kernel) == cudaSuccess) stat = std::max(stat, int(a.sharedSizeBytes));
     if (cudaFuncGetAttributes(&a, build_kernel_pi) == cudaSuccess) stat = std::max(stat, int(a.sharedSizeBytes));
     if (cudaFuncGetAttributes(&a, count_kernel_pi) == cudaSuccess) stat = std::max(stat, int(a.sharedSizeBytes));
-    if (cudaFuncGetAttributes(&a, build_kernel_team) == cudaSuccess) stat = std::max(stat, int(a.sharedSizeBytes));
+    if (cudaFuncGetAttributes(&a, build_kernel_team<false>) == cudaSuccess)
+        stat = std::max(stat, int(a.sharedSizeBytes));
+    if (cudaFuncGetAttributes(&a, build_kernel_team<true>) == cudaSuccess)
+        stat = std::max(stat, int(a.sharedSizeBytes));
     cudaGetLastError();
     return optin - stat;
 }
@@ -2198,7 +2212,10 @@ bool prepare_kernels(int smem) {
     ok &= cudaFuncSetAttribute(count_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) == cudaSuccess;
     ok &= cudaFuncSetAttribute(build_kernel_pi, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) == cudaSuccess;
     ok &= cudaFuncSetAttribute(count_kernel_pi, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) == cudaSuccess;
-    ok &= cudaFuncSetAttribute(build_kernel_team, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) == cudaSuccess;
+    ok &= cudaFuncSetAttribute(build_kernel_team<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) ==
+          cudaSuccess;
+    ok &= cudaFuncSetAttribute(build_kernel_team<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) ==
+          cudaSuccess;
     cudaGetLastError();
     if (ok) granted[d] = smem;
     return ok;
@@ -2238,15 +2255,19 @@ int per_item_fit(int ctas, int threads) {
     return std::min((sm / ctas & ~127) - reserved, kernel_smem_limit()) - int(a.sharedSizeBytes);
 }
 
-int max_ctas_per_sm_teams(const SmemPlan &plan, int teams) {
+int max_ctas_per_sm_teams(SmemPlan &plan, int teams) {
     if (teams < 1 || teams > kMaxTeams || plan.threads % 32 || plan.threads * teams > kMaxTeamBlock) return 0;
-    int a = 0;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&a, build_kernel_team, plan.threads * teams,
-                                                      size_t(plan.total) * teams) != cudaSuccess) {
+    const int nt = plan.threads * teams;
+    const size_t smem = size_t(plan.total) * teams;
+    int a = 0, lean = 0;
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&a, build_kernel_team<false>, nt, smem) != cudaSuccess ||
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&lean, build_kernel_team<true>, nt, smem) != cudaSuccess) {
         cudaGetLastError();
         return 0;
     }
-    return a;
+    const bool take = lean >= 2 * a;
+    plan.mode = take ? plan.mode | kLeanTeam : plan.mode & ~kLeanTeam;
+    return take ? lean : a;
 }
 
 int launch_count_pass(const DevMesh &m, const SmemPlan &plan, const int32_t *ids, int32_t n, int64_t *sizes_out,
@@ -2295,8 +2316,9 @@ int launch_build(const DevMesh &m, const SmemPlan &plan, const WorkItem *items, 
     if (teams > 0) {
         if (plans || gscratch || teams > kMaxTeams || plan.threads * teams > kMaxTeamBlock)
             return int(cudaErrorInvalidValue);
-        build_kernel_team<<<grid, plan.threads * teams, size_t(plan.total) * teams, s>>>(m, plan, items, order, n, err,
-                                                                                        ticket, plan.threads);
+        const auto kernel = (plan.mode & kLeanTeam) ? build_kernel_team<true> : build_kernel_team<false>;
+        kernel<<<grid, plan.threads * teams, size_t(plan.total) * teams, s>>>(m, plan, items, order, n, err, ticket,
+                                                                             plan.threads);
     } else if (plans) build_kernel_pi<<<grid, plan.threads, plan.total, s>>>(m, plans, items, order, n, err, ticket);
     else if (gscratch) build_kernel<true><<<grid, plan.threads, 0, s>>>(m, plan, items, order, n, err, ticket, gscratch);
     else build_kernel<false><<<grid, plan.threads, plan.total, s>>>(m, plan, items, order, n, err, ticket, nullptr);
