@@ -227,7 +227,11 @@ gale_status plan_bins(gale_ctx *ctx, bool with_sizes) {
         for (auto &b : ctx->bins) {
             const bool lone_tight = !b.spill && (b.plan.mode & gale::kTight) && ntop[Key(b.plan.threads, b.cut)] < 2;
             if (b.tt_general || lone_tight) {  // each member under its own plan, in build_kernel_pi
-                for (int32_t k : b.clusters) ctx->h_plans[k] = plan_k(k, b.plan.threads);
+                b.plan.total = 0;  // the launch's: what the largest member takes (the bin's plan may take less)
+                for (int32_t k : b.clusters) {
+                    ctx->h_plans[k] = plan_k(k, b.plan.threads);
+                    b.plan.total = std::max(b.plan.total, ctx->h_plans[k].total);
+                }
                 b.per_item = true;
                 kept.push_back(std::move(b));
                 continue;

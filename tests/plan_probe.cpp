@@ -101,6 +101,17 @@ void probe_merged_ctas(gale_ctx *ctx, int32_t total, int32_t *out) {
     out[1] = max_ctas_per_sm(p, false, true);
 }
 
+// per-item bins, and the bytes that some member's own plan takes beyond its
+// launch's shared memory (0: none)
+void probe_per_item(gale_ctx *ctx, int64_t *out) {
+    out[0] = out[1] = 0;
+    for (const Bin &b : ctx->bins) {
+        if (!b.per_item) continue;
+        ++out[0];
+        for (int32_t k : b.clusters) out[1] = std::max<int64_t>(out[1], ctx->h_plans[k].total - b.plan.total);
+    }
+}
+
 int32_t probe_bin_streams(gale_ctx *ctx) { return int32_t(ctx->bin_streams.size()); }
 
 // shared memory of one plan over the listed items (a size bin's)

@@ -88,6 +88,47 @@ def test_list_with_the_largest_member_in_a_fresh_process():
     assert r.returncode == 0, r.stderr[-3000:]
 
 
+def with_third_tets(m, clusters):
+    """m with one more vertex per listed cluster, on a triangle between two of
+    its internal tets: the triangle then lies in three tets."""
+    tv, seg, xyz = [m.tv], [m.seg], [m.xyz]
+    own = (m.seg[m.tv] == np.arange(m.nclusters)[:, None, None]).all(2)
+    for i, k in enumerate(clusters):
+        inside = m.tv[own[k]]
+        faces = np.sort(inside[:, [[1, 2, 3], [0, 2, 3], [0, 1, 3], [0, 1, 2]]].reshape(-1, 3), 1)
+        f, n = np.unique(faces, axis=0, return_counts=True)
+        tv.append([[*f[np.argmax(n == 2)], m.nv + i]])
+        seg.append([k])
+        xyz.append(m.xyz[f[np.argmax(n == 2)]].mean(0, keepdims=True))
+    return gen.Mesh(np.concatenate(xyz), np.concatenate(tv).astype(np.int32), np.concatenate(seg).astype(np.int32),
+                    m.nclusters)
+
+
+def test_non_manifold_members_can_take_more_than_their_bin():
+    m = two_boxes()
+    with gale.Context.load(with_third_tets(m, [m.nclusters - 2, m.nclusters - 1]), device=-1, part_vertices=-1) as ctx:
+        p, big, starred = item_plans(ctx, 512), ctx.K - 2, ctx.K - 1
+        assert merged_total(ctx, [big, starred], 512) < p["total"][big]
+
+
+@pytest.mark.gpu
+def test_per_item_launches_hold_their_largest_member():
+    """Non-manifold clusters share a per-item bin, whose launch has to take
+    the largest member's own plan."""
+    m = two_boxes()
+    m = with_third_tets(m, [m.nclusters - 2, m.nclusters - 1])
+    canon, rel = oracle.build_all(m.nv, m.tv, m.seg, m.nclusters)
+    out = (ctypes.c_int64 * 2)()
+    with gale.Context.load(m, device=0, part_vertices=-1) as ctx:
+        for threads in (0, 256, 1024):
+            ctx.set_tuning(threads)
+            probe().probe_per_item(ctx._h, out)
+            assert out[0] >= 1 and out[1] == 0
+            ctx.build(None, gale.ALL, gale.MODE_BATCHED)
+            ctx.synchronize()
+            assert_bulk_equal(ctx.export(gale.ALL), expected_bulk(rel, canon, range(m.nclusters)))
+
+
 @pytest.mark.gpu
 def test_planned_occupancy_is_the_devices():
     """The kernel's static shared memory counts: two CTAs of 115,200 bytes
